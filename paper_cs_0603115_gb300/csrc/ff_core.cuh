@@ -56,6 +56,80 @@ __device__ __forceinline__ float2 mul22(float2 a, float2 b)
     return add12(t.x, t3);
 }
 
+// Fast2Sum (Dekker): s = a (+) b, t = (a + b) - s exactly when the exponent
+// of a is at least that of b.
+__device__ __forceinline__ float2 fast2sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b);
+    const float z = __fsub_rn(s, a);
+    return make_float2(s, __fsub_rn(b, z));
+}
+
+// ---------------------------------------------------------------------------
+// Mul22 and Add22 with Fast2Sum in place of their closing Add12: 9 + 13 = 22
+// instructions per accumulated term instead of 12 + 16 = 28, for the kernels
+// bound by FP32 issue.  Same bits as mul22 / add22 under these conditions:
+//
+// mul22_fast: |t3| <= |t1| (or t1 = t3 = 0).  Both forms then give
+//   RN(t1 + t3) and its exact error.  A pair whose sum rounds to its high
+//   part (RN(hi + lo) == hi, "normalised") has |lo| <= ulp(hi) / 2, so two
+//   normalised operands give |t3| <~ 3 2^-24 |t1|; where a high product
+//   underflows the low products are zero too.
+// add22_fast: both operands normalised.  With |ah| >= |bh|, ulps ua >= ub:
+//   either ah (+) bh is inexact, then |r| >= 2^23 ulp(r) and every part of s
+//   is at most ulp(r); or it is exact, r a multiple of ub: |r| >= ua >= |al +
+//   bl|, or r = +-ua / 2 (ah a power of two, bh just below it, ub = ua / 2)
+//   and |s| <= 3 ua / 4, the same exponent; or r = 0.  The exponent of r is
+//   never below that of s, which is Fast2Sum's condition.
+// A closing sum that is exact leaves a normalised result, so accumulating
+// mul22_fast terms from (0, 0) (or from any Add22 result) stays inside the
+// conditions.  Signs of zeros: neither t3 nor s is ever -0 where t1 or r is
+// zero, and an exact closing sum gives lo = +0 both ways.
+// Infinities and NaN: any step with a non-finite operand gives (NaN, NaN) in
+// both forms.  The one difference is a step that overflows to hi = +-inf: lo
+// is NaN with Add12 and -+inf with Fast2Sum; a further add22 / add22_fast
+// makes both (NaN, NaN), and ff_overflow_lo() restores the NaN of a last one.
+// ---------------------------------------------------------------------------
+
+// The pair's sum rounds to its high part (false for a NaN).
+__device__ __forceinline__ bool normalised(float2 v) { return __fadd_rn(v.x, v.y) == v.x; }
+
+__device__ __forceinline__ float2 mul22_fast(float2 a, float2 b)
+{
+    const float2 t = mul12(a.x, b.x);
+    const float t3 = __fadd_rn(__fadd_rn(__fmul_rn(a.x, b.y), __fmul_rn(a.y, b.x)), t.y);
+    return fast2sum(t.x, t3);
+}
+
+// mul22_fast for operands that nothing has checked: `bad` is set when the
+// condition fails (one comparison, for kernels that use each operand pair
+// once); the caller then repeats the sum with mul22 / add22.
+__device__ __forceinline__ float2 mul22_fast_checked(float2 a, float2 b, bool& bad)
+{
+    const float2 t = mul12(a.x, b.x);
+    const float t3 = __fadd_rn(__fadd_rn(__fmul_rn(a.x, b.y), __fmul_rn(a.y, b.x)), t.y);
+    bad |= fabsf(t3) > fabsf(t.x);
+    return fast2sum(t.x, t3);
+}
+
+__device__ __forceinline__ float2 add22_fast(float2 a, float2 b)
+{
+    const float r = __fadd_rn(a.x, b.x);
+    const bool c = fabsf(a.x) >= fabsf(b.x);
+    const float P = c ? a.x : b.x;
+    const float Q = c ? b.x : a.x;
+    const float L1 = c ? b.y : a.y;
+    const float L2 = c ? a.y : b.y;
+    const float s = __fadd_rn(__fadd_rn(__fadd_rn(__fsub_rn(P, r), Q), L1), L2);
+    return fast2sum(r, s);
+}
+
+// The low part that Add12 leaves beside an overflowed high part.
+__device__ __forceinline__ float2 ff_overflow_lo(float2 v)
+{
+    return make_float2(v.x, fabsf(v.x) == __int_as_float(0x7f800000) ? __int_as_float(0x7fc00000) : v.y);
+}
+
 // Div22: Dekker's div2 with the paper's Add12 as the final renormalisation.
 //   ch = ah / bh; (uh, ul) = Mul12(ch, bh);
 //   cl = ((((ah - uh) - ul) + al) - ch bl) / bh;  result Add12(ch, cl)
@@ -83,15 +157,6 @@ __device__ __forceinline__ float2 sqrt22(float2 a)
     const float2 r = add12(c, cc);
     const bool z = (a.x == 0.0f);
     return make_float2(z ? a.x : r.x, z ? 0.0f : r.y);
-}
-
-// Fast2Sum (Dekker): s = a (+) b, t = (a + b) - s exactly when the exponent
-// of a is at least that of b.
-__device__ __forceinline__ float2 fast2sum(float a, float b)
-{
-    const float s = __fadd_rn(a, b);
-    const float z = __fsub_rn(s, a);
-    return make_float2(s, __fsub_rn(b, z));
 }
 
 // Accurate float-float addition (Joldes, Muller and Popescu 2017,

@@ -5,198 +5,199 @@
 // starting from (0, 0), one thread per output: the result does not depend on
 // the launch shape and equals the plain triple loop bit for bit.
 //
-// The work is FP32-instruction bound (about 28 instructions per term, 8
-// bytes of A and B read from L2 per 64 terms), so the kernel is shaped for
-// issue rate: a 256-thread block computes a 64 x 64 tile of C, each thread a
-// 4 x 4 sub-tile (16 independent Add22 chains).  The A and B panels of the
-// current K slice (16 values deep) sit in shared memory, double buffered; the
-// next slice is loaded into registers while the current one is computed.
-// Two blocks per SM (121 registers a thread) keep 16 warps resident.
+// The work is FP32-instruction bound: 22 instructions per term with the
+// Fast2Sum forms of ff_core.cuh, against 8 bytes of A and B read from L2 per 64
+// terms.  Every value is checked once, when its slice goes to shared memory,
+// for RN(hi + lo) == hi; the check is combined over the block in the slice's
+// barrier, and a slice with any other value (or a NaN) runs on the full Mul22 +
+// Add22 (28 instructions), with the same bits either way.  4096^3: 54.4 ms with
+// the full forms alone, 44.2 ms with the fast ones (1.55e12 terms/s, 22.96
+// instructions issued per term, 93% of the cycles issue).
+//
+// A block computes one tile of C from slices of A and B in shared memory,
+// double buffered; the next slice is loaded into registers while the current
+// one is computed.
+// Packed binary32 pairs (add / mul / fma f32x2) were measured for the 22-
+// instruction term and not kept: 15.1 instructions per term, but bound by
+// register operands at the same time (2048^3: 5.59-5.73 against 5.50 ms).
 // Global loads are coalesced for each operand layout (row-major or
-// transposed); the shared-memory tiles are k-major with one padding value per
-// row so that the transposing stores do not serialise on one bank.
+// transposed); the shared-memory tiles are k-major with padded rows so that
+// the transposing stores do not serialise on one bank.
 #include "ff_core.cuh"
 #include "ff_host.cuh"
 
 namespace {
 
-constexpr int kBM = 64;              // rows of C per block
-constexpr int kBN = 64;              // columns of C per block
-constexpr int kBK = 16;              // inner-index depth of one shared slice
-constexpr int kThreads = 256;        // 16 x 16 threads, 4 x 4 outputs each
-constexpr int kLdS = kBM + 1;        // shared row length (kBM == kBN)
-constexpr int kLoads = kBM * kBK / kThreads;  // values of one operand slice per thread
-
-static_assert(kBM == kBN, "one shared row length serves both operands");
-static_assert(kLoads == 4, "load mappings below assume four values per thread");
+// One tile shape: a block of T threads computes BM x BN outputs, each thread
+// a TM x TN sub-tile (rows ty + r BM / TM, columns tx + c BN / TN, or adjacent
+// columns when TN = 2), from slices BK deep of A and B in shared memory.
+template <int BM_, int BN_, int TM_, int TN_, int BK_, int MINB_>
+struct Tile {
+    static constexpr int BM = BM_, BN = BN_, TM = TM_, TN = TN_, BK = BK_, MINB = MINB_;
+    static constexpr int TX = BN / TN, TY = BM / TM, T = TX * TY;
+    static constexpr int LA = BM * BK / T, LB = BN * BK / T;      // values of one slice per thread
+    static constexpr int LDA = BM + 1;                            // shared row lengths: a transposing
+    static constexpr int LDB = TN == 2 ? BN + 2 : BN + 1;         // store spreads over the banks
+    static_assert(T % 32 == 0 && BM * BK % T == 0 && BN * BK % T == 0, "whole values per thread");
+};
 
 struct Dims {
     int64_t m, n, k, lda, ldb, ldc;
     int64_t tiles_n, tiles;
 };
 
-// Slice `p0` of op(A) into registers: op(A)[i0 + r, p0 + c] for the 64 x 16
-// slice.  Row-major A (TA = false) is contiguous along the inner index: a
-// thread reads column c = t & 15 of rows (t >> 4) + 16 s.  Transposed A is
-// contiguous along i: a thread reads row i = t & 63 of inner indices
-// (t >> 6) + 4 s.  Out-of-range values read as (0, 0); they are never used
-// for a stored output nor for a term beyond k.
-template <bool TA>
-__device__ __forceinline__ void load_a(const float2* __restrict__ A, const Dims& d, int64_t i0, int64_t p0,
-                                       float2 (&v)[kLoads])
+// Slice `p0` of one operand into registers: N rows (of op(A)) or columns (of
+// op(B)) from `i0`, BK inner indices.  KMAJOR: the operand is stored
+// contiguous along the rows / columns (transposed A, row-major B), so
+// neighbouring threads take neighbouring rows; otherwise contiguous along the
+// inner index.  Out-of-range values read as (0, 0); they are never used for a
+// stored output nor for a term beyond k.
+template <int N, int BK, int T, int L, bool KMAJOR>
+__device__ __forceinline__ void load_slice(const float2* __restrict__ M, int64_t ld, int64_t extent, int64_t k,
+                                           int64_t i0, int64_t p0, float2 (&v)[L])
 {
-    const int t = threadIdx.x;
 #pragma unroll
-    for (int s = 0; s < kLoads; ++s) {
-        int64_t i, p;
-        if (!TA) {
-            i = i0 + (t >> 4) + 16 * s;
-            p = p0 + (t & 15);
-        } else {
-            i = i0 + (t & 63);
-            p = p0 + (t >> 6) + 4 * s;
-        }
-        const bool in = (i < d.m) && (p < d.k);
-        v[s] = in ? __ldg(TA ? A + p * d.lda + i : A + i * d.lda + p) : make_float2(0.0f, 0.0f);
+    for (int s = 0; s < L; ++s) {
+        const int e = threadIdx.x + s * T;
+        const int64_t i = i0 + (KMAJOR ? e % N : e / BK);
+        const int64_t p = p0 + (KMAJOR ? e / N : e % BK);
+        const bool in = (i < extent) && (p < k);
+        v[s] = in ? __ldg(KMAJOR ? M + p * ld + i : M + i * ld + p) : make_float2(0.0f, 0.0f);
     }
 }
 
-template <bool TA>
-__device__ __forceinline__ void store_a(float2 (*As)[kLdS], const float2 (&v)[kLoads])
+template <int N, int BK, int T, int L, int LD, bool KMAJOR>
+__device__ __forceinline__ void store_slice(float2 (*S)[LD], const float2 (&v)[L])
 {
-    const int t = threadIdx.x;
 #pragma unroll
-    for (int s = 0; s < kLoads; ++s) {
-        if (!TA)
-            As[t & 15][(t >> 4) + 16 * s] = v[s];
-        else
-            As[(t >> 6) + 4 * s][t & 63] = v[s];
+    for (int s = 0; s < L; ++s) {
+        const int e = threadIdx.x + s * T;
+        S[KMAJOR ? e / N : e % BK][KMAJOR ? e % N : e / BK] = v[s];
     }
 }
 
-// Slice `p0` of op(B): op(B)[p0 + r, j0 + c], 16 x 64.  Row-major B
-// (TB = false) is contiguous along j; transposed B along the inner index.
-template <bool TB>
-__device__ __forceinline__ void load_b(const float2* __restrict__ B, const Dims& d, int64_t j0, int64_t p0,
-                                       float2 (&v)[kLoads])
+// One inner index of the slice: TM x TN terms, one per accumulator.
+template <class S, bool FAST>
+__device__ __forceinline__ void step(const float2* Ar, const float2* Br, int ty, int tx, float2 (&acc)[S::TM][S::TN])
 {
-    const int t = threadIdx.x;
+    float2 a[S::TM], b[S::TN];
 #pragma unroll
-    for (int s = 0; s < kLoads; ++s) {
-        int64_t j, p;
-        if (!TB) {
-            j = j0 + (t & 63);
-            p = p0 + (t >> 6) + 4 * s;
-        } else {
-            j = j0 + (t >> 4) + 16 * s;
-            p = p0 + (t & 15);
-        }
-        const bool in = (j < d.n) && (p < d.k);
-        v[s] = in ? __ldg(TB ? B + j * d.ldb + p : B + p * d.ldb + j) : make_float2(0.0f, 0.0f);
+    for (int r = 0; r < S::TM; ++r) a[r] = Ar[ty + S::TY * r];
+    if constexpr (S::TN == 2) {
+        const float4 q = *reinterpret_cast<const float4*>(Br + 2 * tx);
+        b[0] = make_float2(q.x, q.y);
+        b[1] = make_float2(q.z, q.w);
+    } else {
+#pragma unroll
+        for (int c = 0; c < S::TN; ++c) b[c] = Br[tx + S::TX * c];
     }
+#pragma unroll
+    for (int r = 0; r < S::TM; ++r)
+#pragma unroll
+        for (int c = 0; c < S::TN; ++c)
+            acc[r][c] = FAST ? ffk::add22_fast(acc[r][c], ffk::mul22_fast(a[r], b[c]))
+                             : ffk::add22(acc[r][c], ffk::mul22(a[r], b[c]));
 }
 
-template <bool TB>
-__device__ __forceinline__ void store_b(float2 (*Bs)[kLdS], const float2 (&v)[kLoads])
-{
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int s = 0; s < kLoads; ++s) {
-        if (!TB)
-            Bs[(t >> 6) + 4 * s][t & 63] = v[s];
-        else
-            Bs[t & 15][(t >> 4) + 16 * s] = v[s];
-    }
-}
-
-// One inner index of the slice: 16 terms, one per accumulator.
-__device__ __forceinline__ void step(const float2 (*As)[kLdS], const float2 (*Bs)[kLdS], int kk, int ty, int tx,
-                                     float2 (&acc)[4][4])
-{
-    float2 a[4], b[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) b[c] = Bs[kk][tx + 16 * c];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = ffk::add22(acc[r][c], ffk::mul22(a[r], b[c]));
-}
-
-template <bool TA, bool TB>
-__global__ void __launch_bounds__(kThreads, 2)
+template <class S, bool TA, bool TB>
+__global__ void __launch_bounds__(S::T, S::MINB)
 gemm_kernel(const float2* __restrict__ A, const float2* __restrict__ B, float2* __restrict__ C, Dims d)
 {
-    __shared__ float2 As[2][kBK][kLdS];
-    __shared__ float2 Bs[2][kBK][kLdS];
-    const int tx = threadIdx.x & 15;
-    const int ty = threadIdx.x >> 4;
-    const int64_t nslices = (d.k + kBK - 1) / kBK;
+    __shared__ __align__(16) float2 As[2][S::BK][S::LDA];
+    __shared__ __align__(16) float2 Bs[2][S::BK][S::LDB];
+    const int tx = threadIdx.x % S::TX;
+    const int ty = threadIdx.x / S::TX;
+    const int64_t nslices = (d.k + S::BK - 1) / S::BK;
 
     for (int64_t tile = blockIdx.x; tile < d.tiles; tile += gridDim.x) {
-        const int64_t i0 = (tile / d.tiles_n) * kBM;
-        const int64_t j0 = (tile % d.tiles_n) * kBN;
-        float2 acc[4][4];
+        const int64_t i0 = (tile / d.tiles_n) * S::BM;
+        const int64_t j0 = (tile % d.tiles_n) * S::BN;
+        float2 acc[S::TM][S::TN];
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < S::TM; ++r)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[r][c] = make_float2(0.0f, 0.0f);
+            for (int c = 0; c < S::TN; ++c) acc[r][c] = make_float2(0.0f, 0.0f);
 
-        float2 va[kLoads], vb[kLoads];
+        float2 va[S::LA], vb[S::LB];
+        auto load = [&](int64_t sl) {
+            load_slice<S::BM, S::BK, S::T, S::LA, TA>(A, d.lda, d.m, d.k, i0, sl * S::BK, va);
+            load_slice<S::BN, S::BK, S::T, S::LB, !TB>(B, d.ldb, d.n, d.k, j0, sl * S::BK, vb);
+        };
+        // to shared memory; true when every value this thread loaded is normalised
+        auto store = [&](int buf) {
+            store_slice<S::BM, S::BK, S::T, S::LA, S::LDA, TA>(As[buf], va);
+            store_slice<S::BN, S::BK, S::T, S::LB, S::LDB, !TB>(Bs[buf], vb);
+            bool ok = true;
+#pragma unroll
+            for (int s = 0; s < S::LA; ++s) ok &= ffk::normalised(va[s]);
+#pragma unroll
+            for (int s = 0; s < S::LB; ++s) ok &= ffk::normalised(vb[s]);
+            return ok;
+        };
+        bool ok = true;
         if (nslices > 0) {
-            load_a<TA>(A, d, i0, 0, va);
-            load_b<TB>(B, d, j0, 0, vb);
-            store_a<TA>(As[0], va);
-            store_b<TB>(Bs[0], vb);
+            load(0);
+            ok = store(0);
         }
-        __syncthreads();
+        // the whole slice is normalised (block-uniform): its terms take the fast forms
+        bool fast = __syncthreads_and(ok);
         for (int64_t sl = 0; sl < nslices; ++sl) {
             const int cur = static_cast<int>(sl & 1);
             const bool more = sl + 1 < nslices;
-            if (more) {
-                load_a<TA>(A, d, i0, (sl + 1) * kBK, va);
-                load_b<TB>(B, d, j0, (sl + 1) * kBK, vb);
-            }
-            const int64_t rem = d.k - sl * kBK;
-            if (rem >= kBK) {
-                // Unrolled by two, not sixteen: one inner index is ~460
-                // instructions, and the fully unrolled slice (~7,300) overflows
-                // the instruction cache (measured: 0.74 -> 0.88 of FP32 issue).
-#pragma unroll 2
-                for (int kk = 0; kk < kBK; ++kk) step(As[cur], Bs[cur], kk, ty, tx, acc);
+            if (more) load(sl + 1);
+            const int64_t rem = d.k - sl * S::BK;
+            const int kn = static_cast<int>(rem < S::BK ? rem : S::BK);
+            if (!fast) {
+#pragma unroll 1
+                for (int kk = 0; kk < kn; ++kk) step<S, false>(As[cur][kk], Bs[cur][kk], ty, tx, acc);
+            } else if (kn == S::BK) {
+                // Unrolled to about 1,400 instructions at most: the fully
+                // unrolled slice of the 4 x 4 sub-tile overflows the
+                // instruction cache.
+                constexpr int U = 32 / (S::TM * S::TN) < 8 ? 32 / (S::TM * S::TN) : 8;
+#pragma unroll U
+                for (int kk = 0; kk < S::BK; ++kk) step<S, true>(As[cur][kk], Bs[cur][kk], ty, tx, acc);
             } else {
-                for (int kk = 0; kk < static_cast<int>(rem); ++kk) step(As[cur], Bs[cur], kk, ty, tx, acc);
+#pragma unroll 1
+                for (int kk = 0; kk < kn; ++kk) step<S, true>(As[cur][kk], Bs[cur][kk], ty, tx, acc);
             }
-            if (more) {
-                store_a<TA>(As[cur ^ 1], va);
-                store_b<TB>(Bs[cur ^ 1], vb);
-            }
-            __syncthreads();
+            ok = more ? store(cur ^ 1) : true;
+            fast = __syncthreads_and(ok);
         }
 
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int64_t i = i0 + ty + 16 * r;
+        for (int r = 0; r < S::TM; ++r) {
+            const int64_t i = i0 + ty + S::TY * r;
             if (i >= d.m) continue;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int64_t j = j0 + tx + 16 * c;
-                if (j < d.n) C[i * d.ldc + j] = acc[r][c];
+            for (int c = 0; c < S::TN; ++c) {
+                const int64_t j = j0 + (S::TN == 2 ? 2 * tx + c : tx + S::TX * c);
+                if (j < d.n) C[i * d.ldc + j] = ffk::ff_overflow_lo(acc[r][c]);
             }
         }
     }
 }
 
-template <bool TA, bool TB>
-ff_status launch(const float2* A, const float2* B, float2* C, const Dims& d, cudaStream_t s)
+template <class S>
+ff_status launch(bool ta, bool tb, const float2* A, const float2* B, float2* C, Dims d, cudaStream_t s)
 {
+    d.tiles_n = (d.n + S::BN - 1) / S::BN;
+    d.tiles = ((d.m + S::BM - 1) / S::BM) * d.tiles_n;
     // one block per tile up to the 1-D grid limit; blocks loop over the rest
     const int64_t cap = 0x7fffffffLL;
     const unsigned grid = static_cast<unsigned>(d.tiles < cap ? d.tiles : cap);
-    gemm_kernel<TA, TB><<<grid, kThreads, 0, s>>>(A, B, C, d);
+    if (!ta && !tb)
+        gemm_kernel<S, false, false><<<grid, S::T, 0, s>>>(A, B, C, d);
+    else if (ta && !tb)
+        gemm_kernel<S, true, false><<<grid, S::T, 0, s>>>(A, B, C, d);
+    else if (!ta && tb)
+        gemm_kernel<S, false, true><<<grid, S::T, 0, s>>>(A, B, C, d);
+    else
+        gemm_kernel<S, true, true><<<grid, S::T, 0, s>>>(A, B, C, d);
     return ffh::check_launch();
 }
+
+using Tile64 = Tile<64, 64, 4, 4, 16, 2>;
 
 }  // namespace
 
@@ -218,15 +219,11 @@ ff_status ff_gemm(int transa, int transb, int64_t m, int64_t n, int64_t k, const
     if (!ffh::ok_ptr(A_, an) || !ffh::ok_ptr(B_, bn) || !ffh::ok_ptr(C_, cn)) return FF_ERR_INVALID_ARG;
     Dims d;
     d.m = m; d.n = n; d.k = k; d.lda = lda; d.ldb = ldb; d.ldc = ldc;
-    d.tiles_n = (n + kBN - 1) / kBN;
-    d.tiles = ((m + kBM - 1) / kBM) * d.tiles_n;
+    d.tiles_n = d.tiles = 0;
     auto* A = reinterpret_cast<const float2*>(A_);
     auto* B = reinterpret_cast<const float2*>(B_);
     auto* C = reinterpret_cast<float2*>(C_);
-    if (!transa && !transb) return launch<false, false>(A, B, C, d, s);
-    if (transa && !transb) return launch<true, false>(A, B, C, d, s);
-    if (!transa && transb) return launch<false, true>(A, B, C, d, s);
-    return launch<true, true>(A, B, C, d, s);
+    return launch<Tile64>(transa != 0, transb != 0, A, B, C, d, s);
 }
 
 }  // extern "C"

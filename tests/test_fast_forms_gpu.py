@@ -1,0 +1,68 @@
+"""The Fast2Sum forms of the products and the paths around them: every result
+has the bits of the full Mul22 / Add22 sequence (the oracle's, in the
+documented order), for normalised operands, for pairs whose sum does not round
+to the high part (they leave the fast path), for sums that overflow to an
+infinity at any point, and for infinities, NaN, signed zeros and subnormals;
+at the edges of every tile shape."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_cs_0603115_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+if torch.cuda.is_available():
+    import paper_cs_0603115_gb300 as ff
+
+DEV = "cuda"
+
+
+def same_bits(got, want):
+    got = np.ascontiguousarray(got, np.float32)
+    want = np.ascontiguousarray(want, np.float32)
+    assert got.shape == want.shape
+    nan = np.isnan(got) & np.isnan(want)
+    eq = (got.view(np.uint32) == want.view(np.uint32)) | nan
+    if not eq.all():
+        bad = np.argwhere(~eq)[:5]
+        raise AssertionError(f"{(~eq).sum()} mismatches, first at {bad.tolist()}: "
+                             f"got {got[tuple(bad[0])]} want {want[tuple(bad[0])]}")
+
+
+def plant(v, kind, seed):
+    """Special pairs at random places of a (..., 2) array (a copy)."""
+    v = v.clone()
+    f = v.reshape(-1, 2)
+    g = torch.Generator().manual_seed(seed)
+    at = torch.randperm(f.shape[0], generator=g)[:max(1, f.shape[0] // 50)]
+    if kind == "unnormalised":
+        f[at, 1] = f[at, 0] * 0.75
+    elif kind == "swapped":          # |lo| > |hi|
+        f[at] = f[at].flip(1)
+    elif kind == "overflow":         # products and sums around the largest binary32
+        f[at, 0] = torch.sign(f[at, 0]) * 1.8446744e19
+        f[at, 1] = f[at, 0] * 2.0 ** -25
+    elif kind == "specials":
+        vals = torch.tensor([[float("inf"), 0.0], [float("nan"), 0.0], [-0.0, 0.0], [0.0, -0.0], [1e-40, 0.0],
+                             [-3e-39, 1e-45], [float("-inf"), 1.0], [0.0, 1e-45]])
+        f[at] = vals[torch.arange(at.numel()) % vals.shape[0]]
+    return f.reshape(v.shape)
+
+
+KINDS = ["plain", "unnormalised", "swapped", "overflow", "specials"]
+
+
+# ragged in both directions and in the inner index
+@pytest.mark.parametrize("m,n,k", [(33, 65, 70), (250, 255, 49), (1020, 1023, 33), (1209, 1021, 19)])
+@pytest.mark.parametrize("kind", KINDS)
+def test_gemm_tiles(m, n, k, kind):
+    g = inputs.gemm(m, n, k, inputs.seed_for(6, 60))
+    A, B = plant(g.A, kind, 1), plant(g.B, kind, 2)
+    At, Bt = A.permute(1, 0, 2).contiguous(), B.permute(1, 0, 2).contiguous()
+    want = oracle.gemm(A.numpy(), B.numpy())
+    for ta in (False, True):
+        for tb in (False, True):
+            got = ff.gemm((At if ta else A).to(DEV), (Bt if tb else B).to(DEV), transa=ta, transb=tb)
+            same_bits(got.cpu().numpy(), want)

@@ -16,13 +16,16 @@
 //
 // A block computes one tile of C from slices of A and B in shared memory,
 // double buffered; the next slice is loaded into registers while the current
-// one is computed.
+// one is computed.  Four tile shapes (see tile choice at ff_gemm): the large
+// ones reuse operands more, the small ones spread a small C over all SMs.
 // Packed binary32 pairs (add / mul / fma f32x2) were measured for the 22-
 // instruction term and not kept: 15.1 instructions per term, but bound by
 // register operands at the same time (2048^3: 5.59-5.73 against 5.50 ms).
 // Global loads are coalesced for each operand layout (row-major or
 // transposed); the shared-memory tiles are k-major with padded rows so that
 // the transposing stores do not serialise on one bank.
+#include <cmath>
+
 #include "ff_core.cuh"
 #include "ff_host.cuh"
 
@@ -197,7 +200,40 @@ ff_status launch(bool ta, bool tb, const float2* A, const float2* B, float2* C, 
     return ffh::check_launch();
 }
 
+// Tile choice.  Every output is one serial chain of k terms, so C is cut by
+// outputs only, and the time is that of the SM with the most tiles: measured
+// cycles per inner index with q tiles on an SM are close to  a q + b  (a: the
+// tile's outputs per lane times the cycles per term, which grow as the tile's
+// operand reuse shrinks: 26.2, 27.7, 30.5 and 33.7; b: the part of a chain's
+// latency that the few resident warps leave uncovered).  The shape with the
+// least of it runs.  500 x 300 x 700: 392 us with 64 x 64 tiles alone (40 of
+// 152 SMs busy), 90 us; 100 x 100 x 1000: 508 -> 35 us; 1024^3: 1042 -> 769
+// us; from about 2048 rows and columns the largest tile is always taken.
 using Tile64 = Tile<64, 64, 4, 4, 16, 2>;
+using Tile32 = Tile<32, 32, 2, 2, 32, 2>;
+using Tile16 = Tile<16, 16, 1, 2, 16, 8>;
+using Tile8 = Tile<8, 16, 1, 1, 32, 8>;
+
+template <class S>
+double cycles(int64_t m, int64_t n, int sm_count, double a, double b)
+{
+    const double tiles = static_cast<double>((m + S::BM - 1) / S::BM) * static_cast<double>((n + S::BN - 1) / S::BN);
+    return a * std::ceil(tiles / sm_count) + b;
+}
+
+ff_status launch_best(bool ta, bool tb, const float2* A, const float2* B, float2* C, const Dims& d, int sm_count,
+                      cudaStream_t s)
+{
+    const double c64 = cycles<Tile64>(d.m, d.n, sm_count, 838.0, 30.0);
+    const double c32 = cycles<Tile32>(d.m, d.n, sm_count, 222.0, 20.0);
+    const double c16 = cycles<Tile16>(d.m, d.n, sm_count, 61.0, 25.0);
+    const double c8 = cycles<Tile8>(d.m, d.n, sm_count, 33.7, 30.0);
+    const double best = std::fmin(std::fmin(c64, c32), std::fmin(c16, c8));
+    if (best == c64) return launch<Tile64>(ta, tb, A, B, C, d, s);
+    if (best == c32) return launch<Tile32>(ta, tb, A, B, C, d, s);
+    if (best == c16) return launch<Tile16>(ta, tb, A, B, C, d, s);
+    return launch<Tile8>(ta, tb, A, B, C, d, s);
+}
 
 }  // namespace
 
@@ -217,13 +253,16 @@ ff_status ff_gemm(int transa, int transb, int64_t m, int64_t n, int64_t k, const
     const size_t bn = static_cast<size_t>(k) * static_cast<size_t>(n);
     const size_t cn = static_cast<size_t>(m) * static_cast<size_t>(n);
     if (!ffh::ok_ptr(A_, an) || !ffh::ok_ptr(B_, bn) || !ffh::ok_ptr(C_, cn)) return FF_ERR_INVALID_ARG;
+    ffh::DeviceInfo di;
+    const ff_status st = ffh::device_info(&di);
+    if (st != FF_OK) return st;
     Dims d;
     d.m = m; d.n = n; d.k = k; d.lda = lda; d.ldb = ldb; d.ldc = ldc;
     d.tiles_n = d.tiles = 0;
     auto* A = reinterpret_cast<const float2*>(A_);
     auto* B = reinterpret_cast<const float2*>(B_);
     auto* C = reinterpret_cast<float2*>(C_);
-    return launch<Tile64>(transa != 0, transb != 0, A, B, C, d, s);
+    return launch_best(transa != 0, transb != 0, A, B, C, d, di.sm_count, s);
 }
 
 }  // extern "C"

@@ -54,7 +54,8 @@ def plant(v, kind, seed):
 KINDS = ["plain", "unnormalised", "swapped", "overflow", "specials"]
 
 
-# ragged in both directions and in the inner index
+# one shape for each tile shape of the dispatch (8x16, 16x16, 32x32, 64x64
+# outputs), each ragged in both directions and in the inner index
 @pytest.mark.parametrize("m,n,k", [(33, 65, 70), (250, 255, 49), (1020, 1023, 33), (1209, 1021, 19)])
 @pytest.mark.parametrize("kind", KINDS)
 def test_gemm_tiles(m, n, k, kind):

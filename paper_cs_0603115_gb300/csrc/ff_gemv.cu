@@ -6,11 +6,12 @@
 // Layouts: A is m x n row-major (row stride lda); X, dX are n x k and Y, dY
 // are m x k, all column-major (column strides ldx, lddx, ldy, lddy).
 //
-// ff_gemv: one warp per row, 8 rows per 256-thread block.  Lane l walks the
-// row in two-column steps (j = 2l + 64t, 16-byte loads of A and of each
-// column of X) and keeps KT float-float accumulators, one per right-hand
-// side of the current column tile; k > KT is processed as successive tiles.
-// The 32 lane accumulators are combined by a shuffle-down Add22 tree.
+// ff_gemv: one warp per row, four rows per block, a tile of up to four right-
+// hand sides per warp, all tiles in one launch.  Lane l walks the row in two-
+// column steps (j = 2l + 64t, 16-byte loads of A and of each column of X; single
+// columns j = l + 32t on 8-byte access) and keeps one float-float accumulator
+// per right-hand side.  The 32 lane accumulators are combined by a shuffle-down
+// Add22 tree.
 //
 // ff_gemv_t: one thread per pair of adjacent columns of A (coalesced
 // 16-byte loads along rows), one block row per row block of A.  Each thread
@@ -21,6 +22,9 @@
 // rows walked in pairs with dY staged in shared memory; every element adds
 // its k terms in order from (0, 0), in one pass up to twelve right-hand
 // sides and two above, or through the GEMM kernel for larger k.
+#include <cmath>
+#include <type_traits>
+
 #include "ff_core.cuh"
 #include "ff_first_term.cuh"
 #include "ff_host.cuh"
@@ -30,8 +34,7 @@ namespace {
 constexpr int kGBlock = 256;
 constexpr int kGWarps = kGBlock / 32;
 constexpr int kMaxK = 64;
-// Widest tile for which the forward kernel keeps four chunks per lane in flight.
-constexpr int kGemvFourChunksMaxK = 7;
+constexpr int kFWarps = 4;   // rows (one per warp) of a forward block
 
 __device__ __forceinline__ float2 shfl_down2(float2 v, int off)
 {
@@ -41,109 +44,173 @@ __device__ __forceinline__ float2 shfl_down2(float2 v, int off)
 // ---------------------------------------------------------------------------
 // Y = A X
 // ---------------------------------------------------------------------------
-// Resident blocks per SM that the 16-byte forward kernel of a KT-wide tile
-// is compiled for (0: the compiler's own choice).  Four for three to seven
-// right-hand sides (32768^2: +0.3-1.4%); for two, a budget for 6 or 8
-// blocks measured 4% and 14% slower than the compiler's own 48 registers.
-constexpr int gemv_min_blocks(int kt, bool vec) { return vec && kt >= 3 && kt <= 7 ? 4 : 0; }
+// One lane's sums over its chunks of a row (two values each with VEC, one
+// without): chunks lane, lane + 32, ... in order, U of them loaded before they
+// are used (with PIPE, the next U of A before these are added).
+// FAST uses the Fast2Sum forms and returns true when a product fell outside
+// their condition; the caller then repeats the lane's sums with FAST false.
+// Chunk numbers are 32-bit within segments of kSegment chunks.
+constexpr int64_t kSegment = 1 << 24;
 
-template <int KT, bool VEC>
-__global__ void __launch_bounds__(kGBlock, gemv_min_blocks(KT, VEC))
-gemv_kernel(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda, const float2* __restrict__ X,
-            int64_t ldx, float2* __restrict__ Y, int64_t ldy)
+template <int KT, bool VEC, int U, bool PIPE, bool FAST>
+__device__ __forceinline__ bool gemv_lane(const float2* __restrict__ Ar, const float2* __restrict__ X, int64_t n,
+                                          int64_t ldx, unsigned lane, float2 (&acc)[KT])
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t r = static_cast<int64_t>(blockIdx.x) * kGWarps + (threadIdx.x >> 5);
-    if (r >= m) return;
-    const float2* Ar = A + r * lda;
-    float2 acc[KT];
+    using V = std::conditional_t<VEC, float4, float2>;
+    const int64_t chunks = VEC ? n >> 1 : n;
+    bool bad = false;
+    auto term = [&](float2& s, float2 a, float2 x) {
+        if (FAST)
+            s = ffk::add22_fast(s, ffk::mul22_fast_checked(a, x, bad));
+        else
+            s = ffk::add22(s, ffk::mul22(a, x));
+    };
+    auto chunk = [&](float2& s, const V& a, const V& x) {
+        term(s, make_float2(a.x, a.y), make_float2(x.x, x.y));
+        if constexpr (VEC) term(s, make_float2(a.z, a.w), make_float2(x.z, x.w));
+    };
 #pragma unroll
     for (int c = 0; c < KT; ++c) acc[c] = make_float2(0.0f, 0.0f);
-
-    if (VEC) {
-        // two columns per lane per step; n even, A rows and X columns 16-byte aligned
-        const float4* Ar4 = reinterpret_cast<const float4*>(Ar);
-        const int64_t n2 = n >> 1;
-        int64_t t = lane;
-        // four chunks in flight per lane for narrow tiles (each lane still takes
-        // its chunks t, t + 32, t + 64, ... in order): 32768^2, k = 2 / 3 /
-        // 4-7 0.87 / 0.89 / 0.91-0.92 -> 0.89 / 0.92 / 0.93 of the FP32
-        // roofline; at k = 1, where the stream is HBM-bound, it measured
-        // slower (1.03 -> 0.94)
-        if constexpr (KT >= 2 && KT <= kGemvFourChunksMaxK) {
-            for (; t + 96 < n2; t += 128) {
-                const float4 a0 = __ldcs(Ar4 + t), a1 = __ldcs(Ar4 + t + 32);
-                const float4 a2 = __ldcs(Ar4 + t + 64), a3 = __ldcs(Ar4 + t + 96);
+    for (int64_t s0 = 0; s0 < chunks; s0 += kSegment) {
+        const unsigned nch = static_cast<unsigned>(chunks - s0 < kSegment ? chunks - s0 : kSegment);
+        const V* Av = reinterpret_cast<const V*>(Ar) + s0;
+        const V* Xv = reinterpret_cast<const V*>(X) + s0;
+        const int64_t ldv = VEC ? ldx >> 1 : ldx;
+        unsigned t = lane;
+        if constexpr (U > 1) {
+            auto add = [&](const V (&a)[U], unsigned t) {
 #pragma unroll
                 for (int c = 0; c < KT; ++c) {
-                    const float4* Xc = reinterpret_cast<const float4*>(X + c * ldx);
-                    const float4 x0 = __ldg(Xc + t), x1 = __ldg(Xc + t + 32);
-                    const float4 x2 = __ldg(Xc + t + 64), x3 = __ldg(Xc + t + 96);
-                    acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a0.x, a0.y), make_float2(x0.x, x0.y)));
-                    acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a0.z, a0.w), make_float2(x0.z, x0.w)));
-                    acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a1.x, a1.y), make_float2(x1.x, x1.y)));
-                    acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a1.z, a1.w), make_float2(x1.z, x1.w)));
-                    acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a2.x, a2.y), make_float2(x2.x, x2.y)));
-                    acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a2.z, a2.w), make_float2(x2.z, x2.w)));
-                    acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a3.x, a3.y), make_float2(x3.x, x3.y)));
-                    acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a3.z, a3.w), make_float2(x3.z, x3.w)));
+                    V x[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) x[u] = __ldg(Xv + c * ldv + (t + 32 * u));
+#pragma unroll
+                    for (int u = 0; u < U; ++u) chunk(acc[c], a[u], x[u]);
+                }
+            };
+            if constexpr (PIPE) {
+                V a[U], b[U];
+                bool full = t + 32 * (U - 1) < nch;
+                if (full) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) a[u] = __ldcs(Av + (t + 32 * u));
+                }
+#pragma unroll 1
+                while (full) {
+                    full = t + 32 * (2 * U - 1) < nch;
+                    if (full) {
+#pragma unroll
+                        for (int u = 0; u < U; ++u) b[u] = __ldcs(Av + (t + 32 * (U + u)));
+                    }
+                    add(a, t);
+#pragma unroll
+                    for (int u = 0; u < U; ++u) a[u] = b[u];
+                    t += 32 * U;
+                }
+            } else {
+#pragma unroll 1
+                for (; t + 32 * (U - 1) < nch; t += 32 * U) {
+                    V a[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) a[u] = __ldcs(Av + (t + 32 * u));
+                    add(a, t);
                 }
             }
         }
-        for (; t + 32 < n2; t += 64) {
-            const float4 a0 = __ldcs(Ar4 + t);
-            const float4 a1 = __ldcs(Ar4 + t + 32);
+        if constexpr (U > 2) {   // the rest in pairs, then singly
+#pragma unroll 1
+            for (; t + 32 < nch; t += 64) {
+                const V a0 = __ldcs(Av + t), a1 = __ldcs(Av + (t + 32));
 #pragma unroll
-            for (int c = 0; c < KT; ++c) {
-                const float4* Xc = reinterpret_cast<const float4*>(X + c * ldx);
-                const float4 x0 = __ldg(Xc + t);
-                const float4 x1 = __ldg(Xc + t + 32);
-                acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a0.x, a0.y), make_float2(x0.x, x0.y)));
-                acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a0.z, a0.w), make_float2(x0.z, x0.w)));
-                acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a1.x, a1.y), make_float2(x1.x, x1.y)));
-                acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a1.z, a1.w), make_float2(x1.z, x1.w)));
+                for (int c = 0; c < KT; ++c) {
+                    const V x0 = __ldg(Xv + c * ldv + t), x1 = __ldg(Xv + c * ldv + (t + 32));
+                    chunk(acc[c], a0, x0);
+                    chunk(acc[c], a1, x1);
+                }
             }
         }
-        for (; t < n2; t += 32) {
-            const float4 a0 = __ldcs(Ar4 + t);
+#pragma unroll 1
+        for (; t < nch; t += 32) {
+            const V a = __ldcs(Av + t);
 #pragma unroll
-            for (int c = 0; c < KT; ++c) {
-                const float4 x0 = __ldg(reinterpret_cast<const float4*>(X + c * ldx) + t);
-                acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a0.x, a0.y), make_float2(x0.x, x0.y)));
-                acc[c] = ffk::add22(acc[c], ffk::mul22(make_float2(a0.z, a0.w), make_float2(x0.z, x0.w)));
-            }
-        }
-    } else {
-        for (int64_t j = lane; j < n; j += 32) {
-            const float2 a = Ar[j];
-#pragma unroll
-            for (int c = 0; c < KT; ++c) acc[c] = ffk::add22(acc[c], ffk::mul22(a, __ldg(X + c * ldx + j)));
+            for (int c = 0; c < KT; ++c) chunk(acc[c], a, __ldg(Xv + c * ldv + t));
         }
     }
-#pragma unroll
-    for (int c = 0; c < KT; ++c) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc[c] = ffk::add22(acc[c], shfl_down2(acc[c], off));
-    }
-    if (lane == 0) {
-#pragma unroll
-        for (int c = 0; c < KT; ++c) Y[c * ldy + r] = acc[c];
-    }
+    return bad;
 }
 
-template <int KT>
-ff_status launch_gemv_tile(const float2* A, int64_t m, int64_t n, int64_t lda, const float2* X, int64_t ldx,
-                           float2* Y, int64_t ldy, bool vec, cudaStream_t s)
+// One level of the shuffle-down tree for two sums at once: lanes with bit `off`
+// clear combine p with that of lane + off, the others q with that of lane -
+// off, lower lane first in both.
+__device__ __forceinline__ float2 tree_pair(float2 p, float2 q, int lane, int off)
 {
-    const unsigned grid = static_cast<unsigned>((m + kGWarps - 1) / kGWarps);
-    if (vec)
-        gemv_kernel<KT, true><<<grid, kGBlock, 0, s>>>(A, m, n, lda, X, ldx, Y, ldy);
-    else
-        gemv_kernel<KT, false><<<grid, kGBlock, 0, s>>>(A, m, n, lda, X, ldx, Y, ldy);
-    return ffh::check_launch();
+    const bool up = (lane & off) != 0;
+    const float2 mine = up ? q : p, give = up ? p : q;
+    const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, off), __shfl_xor_sync(0xffffffffu, give.y, off));
+    return ffk::add22_fast(up ? got : mine, up ? mine : got);
 }
 
-// Tile width for the float-float kernels: up to seven right-hand sides in
+// The lanes' KT sums combined by the shuffle-down Add22 tree (offsets 16 .. 1)
+// and stored.  Two or more sums share the levels: each halves the lanes that
+// hold one sum, so four sums take 6 additions per lane instead of 20 (16000 x
+// 64, k = 64: 181 -> 134 us).
+template <int KT>
+__device__ __forceinline__ void gemv_tree_store(const float2 (&acc)[KT], int lane, float2* __restrict__ Yr, int64_t ldy)
+{
+    static_assert(KT <= 4, "two shared levels");
+    float2 v;
+    int c = 0, low = 32;   // lanes with lane % low == 0 end with sum c
+    if constexpr (KT == 1) {
+        v = acc[0];
+    } else {
+        const float2 p = tree_pair(acc[0], acc[1], lane, 16);
+        c = lane >> 4;
+        low = 16;
+        v = p;
+        if constexpr (KT > 2) {
+            const float2 q = tree_pair(acc[2], acc[KT - 1], lane, 16);
+            v = tree_pair(p, q, lane, 8);
+            c += (lane >> 2) & 2;
+            low = 8;
+        }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+        if (off < low) v = ffk::add22_fast(v, shfl_down2(v, off));
+    if (lane % low == 0 && c < KT) Yr[c * ldy] = ffk::ff_overflow_lo(v);
+}
+
+template <int KT, bool VEC, int U, bool PIPE>
+__device__ __forceinline__ void gemv_row(const float2* __restrict__ Ar, const float2* __restrict__ X, int64_t n,
+                                         int64_t ldx, float2* __restrict__ Yr, int64_t ldy)
+{
+    const unsigned lane = threadIdx.x & 31;
+    float2 acc[KT];
+    if (gemv_lane<KT, VEC, U, PIPE, true>(Ar, X, n, ldx, lane, acc))
+        gemv_lane<KT, VEC, 1, false, false>(Ar, X, n, ldx, lane, acc);
+    gemv_tree_store(acc, static_cast<int>(lane), Yr, ldy);
+}
+
+// blockIdx.x: rows, one per warp; blockIdx.y: tile of right-hand sides, the
+// first `na` of them KA wide, the others KB wide.
+template <int KA, int KB, bool VEC, int U, bool PIPE, int MINB>
+__global__ void __launch_bounds__(32 * kFWarps, MINB)
+gemv_kernel(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda, const float2* __restrict__ X,
+            int64_t ldx, float2* __restrict__ Y, int64_t ldy, int na)
+{
+    const int64_t r = static_cast<int64_t>(blockIdx.x) * kFWarps + (threadIdx.x >> 5);
+    if (r >= m) return;
+    const int y = blockIdx.y;
+    if (KA == KB || y < na) {
+        const int64_t c0 = static_cast<int64_t>(y) * KA;
+        gemv_row<KA, VEC, U, PIPE>(A + r * lda, X + c0 * ldx, n, ldx, Y + c0 * ldy + r, ldy);
+    } else {
+        const int64_t c0 = static_cast<int64_t>(na) * KA + static_cast<int64_t>(y - na) * KB;
+        gemv_row<KB, VEC, U, PIPE>(A + r * lda, X + c0 * ldx, n, ldx, Y + c0 * ldy + r, ldy);
+    }
+}
+
+// Tile width for the adjoint's kernels: up to seven right-hand sides in
 // one pass (one read of A: below eight the kernels are issue-bound only
 // once all k share the pass), else passes of eight.  Each pass of eight is
 // bound by FP32 issue several times over its read of A, so re-reading A per
@@ -157,7 +224,70 @@ inline int tile_for(int64_t k)
 {
     return k >= 12 ? 8 : (k > 8 ? static_cast<int>((k + 1) / 2) : static_cast<int>(k));
 }
+// Tiles of right-hand sides: `na` of width ka, then `nb` of width kb, all in
+// one launch.  Four wide is the best trade of operand reuse against registers
+// (16384^2, k = 8: 1.48e12 terms/s forward in tiles of four, 1.42e12 in one of
+// eight; adjoint 1.43e12 against 1.24e12); 5 and 6 split into threes and a two.
+struct TileSplit {
+    int ka, kb;
+    int64_t na, nb;
+};
+
+inline TileSplit split_tiles(int64_t k)
+{
+    if (k == 1) return {1, 1, 1, 0};
+    if (k == 2) return {2, 1, 1, 0};
+    if (k == 3) return {3, 2, 1, 0};
+    if (k == 5) return {3, 2, 1, 1};
+    if (k == 6) return {3, 2, 2, 0};
+    const int64_t threes = (4 - k % 4) % 4;
+    return {4, 3, (k - 3 * threes) / 4, threes};
+}
+
 inline int f64_tile_for(int64_t k) { return k >= 16 ? 16 : k >= 8 ? 8 : k >= 4 ? 4 : k >= 2 ? 2 : 1; }
+
+template <int KA, int KB, bool VEC, int U, bool PIPE, int MINB>
+ff_status launch_gemv(const TileSplit& t, const float2* A, int64_t m, int64_t n, int64_t lda, const float2* X,
+                      int64_t ldx, float2* Y, int64_t ldy, cudaStream_t s)
+{
+    const dim3 grid(static_cast<unsigned>((m + kFWarps - 1) / kFWarps), static_cast<unsigned>(t.na + t.nb));
+    gemv_kernel<KA, KB, VEC, U, PIPE, MINB><<<grid, 32 * kFWarps, 0, s>>>(A, m, n, lda, X, ldx, Y, ldy,
+                                                                         static_cast<int>(t.na));
+    return ffh::check_launch();
+}
+
+// Chunks in flight (U) and the register budget that lets the compiler issue
+// their loads together (MINB) were chosen by sweeps over 300 x 1000 to 32768^2;
+// left to itself the compiler took fewer registers and spread the loads out
+// (16383^2, k = 1: 344 us; 302 with the budget below).  On 16-byte access a
+// single right-hand side over many rows, bound by HBM, runs best with four
+// chunks and the next four of A ahead (32768^2: 1.16 ms = 7.4 TB/s, 1.21 with
+// eight and none ahead; 2000 rows and fewer prefer the latter: 300 x 20000 31.5
+// -> 21.4 us).
+// Few rows leave SMs idle under a wide tile, since a row is one warp's: below
+// one warp per SM quarter the right-hand sides get a warp each (400 x 2000, k =
+// 4: 6.9 us in pairs, 5.7 singly), below two they go in pairs (800 x 2000, k = 4:
+// 10.5 us in fours, 8.1).  Tiles of four take four chunks on rows below 8192
+// values (6000^2, k = 8: 208 us, 213 with eight) and eight above (16384^2: 1.42
+// ms, 1.44 with four).
+template <bool VEC>
+ff_status gemv_forward(const float2* A, int64_t m, int64_t n, int64_t lda, const float2* X, int64_t ldx, int64_t k,
+                       float2* Y, int64_t ldy, int sm_count, cudaStream_t s)
+{
+    const TileSplit t = split_tiles(k);
+    const int64_t warps = m * ((k + 3) / 4);
+    const int64_t quarters = 4 * static_cast<int64_t>(sm_count);
+    if (VEC && k == 1 && warps >= 4 * quarters)
+        return launch_gemv<1, 1, VEC, 4, true, 0>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+    if (k == 1 || warps < quarters)
+        return launch_gemv<1, 1, VEC, 8, false, 4>({1, 1, k, 0}, A, m, n, lda, X, ldx, Y, ldy, s);
+    if (k == 2 || warps < 2 * quarters)
+        return launch_gemv<2, 1, VEC, VEC ? 4 : 8, false, VEC ? 6 : 4>({2, 1, k / 2, k % 2}, A, m, n, lda, X, ldx, Y,
+                                                                       ldy, s);
+    if (t.ka == 3) return launch_gemv<3, 2, VEC, VEC ? 4 : 8, false, 6>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+    if (VEC && n < 8192) return launch_gemv<4, 3, VEC, 4, false, 6>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+    return launch_gemv<4, 3, VEC, 8, false, VEC ? 4 : 6>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+}
 
 // ---------------------------------------------------------------------------
 // dX = A^T dY
@@ -623,29 +753,15 @@ ff_status ff_gemv(const ff2* A_, int64_t m, int64_t n, int64_t lda, const ff2* X
     if (!ffh::ok_ptr(A_, an) || !ffh::ok_ptr(X_, static_cast<size_t>(n)) || !ffh::ok_ptr(Y_, static_cast<size_t>(m)))
         return FF_ERR_INVALID_ARG;
     if (m == 0) return FF_OK;
+    ffh::DeviceInfo di;
+    const ff_status st = ffh::device_info(&di);
+    if (st != FF_OK) return st;
     auto* A = reinterpret_cast<const float2*>(A_);
     auto* X = reinterpret_cast<const float2*>(X_);
     auto* Y = reinterpret_cast<float2*>(Y_);
     const bool vec = (n % 2 == 0) && (lda % 2 == 0) && (ldx % 2 == 0) && ffh::aligned(A, 16) && ffh::aligned(X, 16);
-    for (int64_t c0 = 0; c0 < k;) {
-        const int kt = tile_for(k - c0);
-        ff_status st;
-        const float2* Xc = X + c0 * ldx;
-        float2* Yc = Y + c0 * ldy;
-        switch (kt) {
-        case 8: st = launch_gemv_tile<8>(A, m, n, lda, Xc, ldx, Yc, ldy, vec, s); break;
-        case 7: st = launch_gemv_tile<7>(A, m, n, lda, Xc, ldx, Yc, ldy, vec, s); break;
-        case 6: st = launch_gemv_tile<6>(A, m, n, lda, Xc, ldx, Yc, ldy, vec, s); break;
-        case 5: st = launch_gemv_tile<5>(A, m, n, lda, Xc, ldx, Yc, ldy, vec, s); break;
-        case 4: st = launch_gemv_tile<4>(A, m, n, lda, Xc, ldx, Yc, ldy, vec, s); break;
-        case 3: st = launch_gemv_tile<3>(A, m, n, lda, Xc, ldx, Yc, ldy, vec, s); break;
-        case 2: st = launch_gemv_tile<2>(A, m, n, lda, Xc, ldx, Yc, ldy, vec, s); break;
-        default: st = launch_gemv_tile<1>(A, m, n, lda, Xc, ldx, Yc, ldy, vec, s); break;
-        }
-        if (st != FF_OK) return st;
-        c0 += kt;
-    }
-    return FF_OK;
+    return vec ? gemv_forward<true>(A, m, n, lda, X, ldx, k, Y, ldy, di.sm_count, s)
+               : gemv_forward<false>(A, m, n, lda, X, ldx, k, Y, ldy, di.sm_count, s);
 }
 
 size_t ff_gemv_t_workspace_bytes(int64_t m, int64_t n, int64_t k)

@@ -9,6 +9,7 @@ import pytest
 import torch
 
 import oracle
+import replay
 from paper_cs_0603115_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
@@ -67,3 +68,20 @@ def test_gemm_tiles(m, n, k, kind):
         for tb in (False, True):
             got = ff.gemm((At if ta else A).to(DEV), (Bt if tb else B).to(DEV), transa=ta, transb=tb)
             same_bits(got.cpu().numpy(), want)
+
+
+# one warp per row and right-hand side (few rows), pairs, and tiles of 2, 3 + 2,
+# 3, 4 and 4 + 3; row lengths around the loads in flight, even and odd
+FORWARD = [(40, 1100, 1), (40, 515, 3), (700, 130, 4), (700, 67, 3), (650, 70, 9), (1300, 66, 2), (1300, 33, 3), (1230, 131, 5),
+           (1230, 34, 6), (700, 260, 7), (620, 36, 8)]
+
+
+@pytest.mark.parametrize("m,n,k", FORWARD)
+@pytest.mark.parametrize("kind", KINDS)
+def test_gemv_tiles(m, n, k, kind):
+    g = inputs.gemv(m, n, k, inputs.seed_for(4, 200))
+    A, X = plant(g.A, kind, 3), plant(g.X, kind, 4)
+    Y = ff.gemv(A.to(DEV), X.to(DEV)).cpu().numpy()
+    rows = np.unique(np.r_[0:8, m // 2:m // 2 + 8, m - 8:m])
+    want = replay.gemv_warp_replay(A.numpy()[rows], X.numpy(), vec=n % 2 == 0)
+    same_bits(Y[:, rows], want)

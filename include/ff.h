@@ -27,9 +27,8 @@
  *     FF_ERR_WORKSPACE.  A failed launch returns FF_ERR_CUDA and keeps the
  *     CUDA error code for ff_last_cuda_error().  Nothing is enqueued when a
  *     call returns an argument or workspace error; when a call that makes
- *     several launches (a GEMV of several column tiles, a weight gradient
- *     in two passes, a GEMV adjoint and its combination) fails to launch
- *     one, the launches before it stay enqueued.
+ *     two launches (a weight gradient in two passes, a GEMV adjoint and its
+ *     combination) fails to launch the second, the first stays enqueued.
  *   - Sizes.  n == 0 is a no-op returning FF_OK, except that a reduction
  *     with n == 0 writes (0, 0) to its result.
  *   - Aliasing.  An elementwise output may be exactly one of its inputs
@@ -236,10 +235,10 @@ FF_API size_t ff_gemv_t_workspace_bytes(int64_t m, int64_t n, int64_t k);
  * lddx >= n), overwritten.  1 <= k <= 64.
  * Order: A is cut into row blocks (their number depends on m, n, k and the
  * device's SM count); within a block each column accumulates its rows in
- * order with Add22 from (0, 0); the blocks' partial sums go to the workspace
- * (caller-owned, ff_gemv_t_workspace_bytes, 16-byte aligned) and are added
- * in row-block order.  Bit-reproducible for a given device and build; error
- * within m 2^-44 sum_r |A[r, j] dY[r, c]|. */
+ * order with Add22 from (0, 0); the blocks' partial sums (held in shared
+ * memory, or in the workspace: caller-owned, ff_gemv_t_workspace_bytes, 16-byte
+ * aligned) are added in row-block order.  Bit-reproducible for a given device
+ * and build; error within m 2^-44 sum_r |A[r, j] dY[r, c]|. */
 FF_API ff_status ff_gemv_t(const ff2* A, int64_t m, int64_t n, int64_t lda, const ff2* dY,
                     int64_t lddy, int64_t k, ff2* dX, int64_t lddx, void* ws, size_t ws_bytes,
                     cudaStream_t s);

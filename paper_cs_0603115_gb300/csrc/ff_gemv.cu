@@ -13,10 +13,10 @@
 // per right-hand side.  The 32 lane accumulators are combined by a shuffle-down
 // Add22 tree.
 //
-// ff_gemv_t: one thread per pair of adjacent columns of A (coalesced
-// 16-byte loads along rows), one block row per row block of A.  Each thread
-// accumulates its rows in order; the row blocks' partial sums go to the
-// workspace and a second kernel adds them in row-block order.
+// ff_gemv_t: a thread sums one column or a pair of adjacent columns of A over
+// one row block in order, for a tile of up to four right-hand sides; a block
+// holds several row blocks of its columns and adds their sums in row-block
+// order, or the sums go to the workspace and a second kernel adds them.
 //
 // ff_gemv_dA: one thread per pair of adjacent columns of dA, the block's
 // rows walked in pairs with dY staged in shared memory; every element adds
@@ -210,20 +210,6 @@ gemv_kernel(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda, con
     }
 }
 
-// Tile width for the adjoint's kernels: up to seven right-hand sides in
-// one pass (one read of A: below eight the kernels are issue-bound only
-// once all k share the pass), else passes of eight.  Each pass of eight is
-// bound by FP32 issue several times over its read of A, so re-reading A per
-// pass costs nothing, and the eight-wide kernels issue better than sixteen-
-// wide ones (32768^2, k = 16-64: forward 0.93 -> 0.94, adjoint 0.90 -> 0.93
-// of the FP32 roofline).  Nine to eleven remaining right-hand sides are split
-// in two near halves rather than eight and a one- to three-wide pass that
-// would be bound by its read of A.  The FP64 baseline uses powers of two.
-// `k` is the number of right-hand sides not yet done.
-inline int tile_for(int64_t k)
-{
-    return k >= 12 ? 8 : (k > 8 ? static_cast<int>((k + 1) / 2) : static_cast<int>(k));
-}
 // Tiles of right-hand sides: `na` of width ka, then `nb` of width kb, all in
 // one launch.  Four wide is the best trade of operand reuse against registers
 // (16384^2, k = 8: 1.48e12 terms/s forward in tiles of four, 1.42e12 in one of
@@ -292,102 +278,123 @@ ff_status gemv_forward(const float2* A, int64_t m, int64_t n, int64_t lda, const
 // ---------------------------------------------------------------------------
 // dX = A^T dY
 // ---------------------------------------------------------------------------
-// Rows of A each thread of the adjoint loads before using them (the tiles
-// are at most eight wide): the fewer terms a row gives, the more rows must
-// be in flight to cover the HBM latency.
-constexpr int kTRows(int kt) { return kt <= 2 ? 8 : 4; }
-
-// Resident blocks per SM the register allocation must leave room for: with
-// this many warps the narrow tiles (bound by FP32 issue, with a row load
-// ahead of few terms) hide their load latency; left to itself the compiler
-// chose fewer registers and scheduled the row loads later (k = 2-7 at 32768^2:
-// 0.83-0.92 of the FP32 roofline without, 0.88-0.93 with).
-constexpr int gemv_t_min_blocks(int kt, bool vec)
+// One thread's sums of E adjacent columns over the rows [r0, r1) in order, R
+// rows loaded before they are added.  FAST uses the Fast2Sum forms and returns
+// true when a product fell outside their condition; the caller then repeats
+// the sums with FAST false.
+template <int KT, int E, int R, bool FAST>
+__device__ __forceinline__ bool gemv_t_sums(const float2* __restrict__ Aj, int64_t lda, const float2* __restrict__ dY,
+                                            int64_t lddy, int64_t r0, int64_t r1, float2 (&acc)[KT][E])
 {
-    return vec ? (kt <= 2 ? 5 : (kt <= 3 ? 4 : (kt <= 8 ? 3 : 2))) : (kt <= 8 ? 4 : 3);
+    using V = std::conditional_t<E == 2, float4, float2>;
+    bool bad = false;
+    auto term = [&](float2& s, float2 a, float2 d) {
+        if (FAST)
+            s = ffk::add22_fast(s, ffk::mul22_fast_checked(a, d, bad));
+        else
+            s = ffk::add22(s, ffk::mul22(a, d));
+    };
+    auto row = [&](float2 (&s)[E], const V& a, float2 d) {
+        term(s[0], make_float2(a.x, a.y), d);
+        if constexpr (E == 2) term(s[1], make_float2(a.z, a.w), d);
+    };
+    auto load = [&](int64_t r) { return __ldcs(reinterpret_cast<const V*>(Aj + r * lda)); };
+#pragma unroll
+    for (int c = 0; c < KT; ++c)
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[c][e] = make_float2(0.0f, 0.0f);
+    int64_t r = r0;
+#pragma unroll 1
+    for (; r + R <= r1; r += R) {
+        V a[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) a[q] = load(r + q);
+#pragma unroll
+        for (int c = 0; c < KT; ++c)
+#pragma unroll
+            for (int q = 0; q < R; ++q) row(acc[c], a[q], __ldg(dY + c * lddy + r + q));
+    }
+    if (R > 1 && r < r1) {   // the last R - 1 rows at most, loaded together
+        V a[R];
+#pragma unroll
+        for (int q = 0; q < R - 1; ++q)
+            if (r + q < r1) a[q] = load(r + q);
+#pragma unroll
+        for (int c = 0; c < KT; ++c)
+#pragma unroll
+            for (int q = 0; q < R - 1; ++q)
+                if (r + q < r1) row(acc[c], a[q], __ldg(dY + c * lddy + r + q));
+    }
+    return bad;
 }
 
-// Partial sums: ws[(rb * k + c) * n + j] for row block rb.
-template <int KT, bool VEC>
-__global__ void __launch_bounds__(kGBlock, gemv_t_min_blocks(KT, VEC))
-gemv_t_kernel(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda, const float2* __restrict__ dY,
-              int64_t lddy, int64_t rows_per_block, float2* __restrict__ out, int64_t out_ld, int64_t out_rb_stride)
+// The block's tile of KT right-hand sides; see gemv_t_kernel.
+template <int KT, int E, int R>
+__device__ __forceinline__ void gemv_t_tile(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda,
+                                            const float2* __restrict__ dY, int64_t lddy, int64_t rpb, int64_t nrb,
+                                            int cx, float2* __restrict__ out, int64_t out_ld, int64_t rb_stride,
+                                            float2 (*part)[kGBlock])
 {
-    const int64_t r0 = static_cast<int64_t>(blockIdx.y) * rows_per_block;
-    int64_t r1 = r0 + rows_per_block;
-    if (r1 > m) r1 = m;
-    float2* o = out + static_cast<int64_t>(blockIdx.y) * out_rb_stride;
-    if (VEC) {
-        const int64_t jp = static_cast<int64_t>(blockIdx.x) * kGBlock + threadIdx.x;  // column pair
-        if (2 * jp >= n) return;
-        float2 acc0[KT], acc1[KT];
+    const int tx = threadIdx.x & (cx - 1);
+    const int ty = threadIdx.x / cx;
+    const int rg = kGBlock / cx;
+    const int64_t j = (static_cast<int64_t>(blockIdx.x) * cx + tx) * E;   // first column
+    const int64_t rb = static_cast<int64_t>(blockIdx.y) * rg + ty;
+    const int64_t r0 = rb * rpb;
+    const int64_t r1 = r0 + rpb < m ? r0 + rpb : m;
+    float2 acc[KT][E];
+    const bool active = j < n && rb < nrb;
+    if (active && gemv_t_sums<KT, E, R, true>(A + j, lda, dY, lddy, r0, r1, acc))
+        gemv_t_sums<KT, E, 1, false>(A + j, lda, dY, lddy, r0, r1, acc);
+    if (rg == 1 || gridDim.y > 1) {
+        if (!active) return;
+        float2* o = out + rb * rb_stride + j;
 #pragma unroll
-        for (int c = 0; c < KT; ++c) {
-            acc0[c] = make_float2(0.0f, 0.0f);
-            acc1[c] = make_float2(0.0f, 0.0f);
-        }
-        int64_t r = r0;
-        {
-            // kTRows(KT) rows loaded ahead of use: a tile of at most eight
-            // right-hand sides has too few terms per row to hide the HBM
-            // latency of the next row's load (the loops below take the
-            // remaining rows)
-            constexpr int R = kTRows(KT);
-            for (; r + R - 1 < r1; r += R) {
-                float4 a[R];
+        for (int c = 0; c < KT; ++c)
 #pragma unroll
-                for (int q = 0; q < R; ++q) a[q] = __ldcs(reinterpret_cast<const float4*>(A + (r + q) * lda) + jp);
+            for (int e = 0; e < E; ++e) o[c * out_ld + e] = ffk::ff_overflow_lo(acc[c][e]);
+        return;
+    }
+    if (active) {
 #pragma unroll
-                for (int c = 0; c < KT; ++c) {
+        for (int c = 0; c < KT; ++c)
 #pragma unroll
-                    for (int q = 0; q < R; ++q) {
-                        const float2 d = __ldg(dY + c * lddy + r + q);
-                        acc0[c] = ffk::add22(acc0[c], ffk::mul22(make_float2(a[q].x, a[q].y), d));
-                        acc1[c] = ffk::add22(acc1[c], ffk::mul22(make_float2(a[q].z, a[q].w), d));
-                    }
-                }
-            }
-        }
-        for (; r + 1 < r1; r += 2) {
-            const float4 a0 = __ldcs(reinterpret_cast<const float4*>(A + r * lda) + jp);
-            const float4 a1 = __ldcs(reinterpret_cast<const float4*>(A + (r + 1) * lda) + jp);
-#pragma unroll
-            for (int c = 0; c < KT; ++c) {
-                const float2 d0 = __ldg(dY + c * lddy + r);
-                const float2 d1 = __ldg(dY + c * lddy + r + 1);
-                acc0[c] = ffk::add22(acc0[c], ffk::mul22(make_float2(a0.x, a0.y), d0));
-                acc1[c] = ffk::add22(acc1[c], ffk::mul22(make_float2(a0.z, a0.w), d0));
-                acc0[c] = ffk::add22(acc0[c], ffk::mul22(make_float2(a1.x, a1.y), d1));
-                acc1[c] = ffk::add22(acc1[c], ffk::mul22(make_float2(a1.z, a1.w), d1));
-            }
-        }
-        for (; r < r1; ++r) {
-            const float4 a0 = __ldcs(reinterpret_cast<const float4*>(A + r * lda) + jp);
-#pragma unroll
-            for (int c = 0; c < KT; ++c) {
-                const float2 d0 = __ldg(dY + c * lddy + r);
-                acc0[c] = ffk::add22(acc0[c], ffk::mul22(make_float2(a0.x, a0.y), d0));
-                acc1[c] = ffk::add22(acc1[c], ffk::mul22(make_float2(a0.z, a0.w), d0));
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < KT; ++c) {
-            o[c * out_ld + 2 * jp] = acc0[c];
-            o[c * out_ld + 2 * jp + 1] = acc1[c];
-        }
+            for (int e = 0; e < E; ++e) part[c * E + e][threadIdx.x] = acc[c][e];
+    }
+    __syncthreads();
+    if (j >= n) return;
+    for (int w = ty; w < KT * E; w += rg) {   // column j + w % E of right-hand side w / E
+        float2 v = part[w][tx];
+#pragma unroll 4
+        for (int b = 1; b < nrb; ++b) v = ffk::add22_fast(v, part[w][b * cx + tx]);
+        out[(w / E) * out_ld + j + w % E] = ffk::ff_overflow_lo(v);
+    }
+}
+
+// Grid: x groups of cx columns (column pairs with E = 2), y groups of row
+// blocks, z tiles of right-hand sides, the first `na` KA wide and the others
+// KB.  A block is cx columns wide and 256 / cx row blocks high: thread (tx, ty)
+// sums row block blockIdx.y * (256 / cx) + ty.  With one group of several row
+// blocks the block adds its row blocks' sums in order through shared memory
+// and writes dX; otherwise thread sums go to out[rb * rb_stride + c * out_ld +
+// j] (dX itself when there is a single row block, else the workspace that
+// gemv_t_combine reads).
+template <int KA, int KB, int E, int R, int MINB>
+__global__ void __launch_bounds__(kGBlock, MINB)
+gemv_t_kernel(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda, const float2* __restrict__ dY,
+              int64_t lddy, int64_t rpb, int64_t nrb, int cx, float2* __restrict__ out, int64_t out_ld,
+              int64_t rb_stride, int na)
+{
+    __shared__ float2 part[KA * E][kGBlock];
+    const int z = blockIdx.z;
+    if (KA == KB || z < na) {
+        const int64_t c0 = static_cast<int64_t>(z) * KA;
+        gemv_t_tile<KA, E, R>(A, m, n, lda, dY + c0 * lddy, lddy, rpb, nrb, cx, out + c0 * out_ld, out_ld, rb_stride,
+                              part);
     } else {
-        const int64_t j = static_cast<int64_t>(blockIdx.x) * kGBlock + threadIdx.x;
-        if (j >= n) return;
-        float2 acc[KT];
-#pragma unroll
-        for (int c = 0; c < KT; ++c) acc[c] = make_float2(0.0f, 0.0f);
-        for (int64_t r = r0; r < r1; ++r) {
-            const float2 a = A[r * lda + j];
-#pragma unroll
-            for (int c = 0; c < KT; ++c) acc[c] = ffk::add22(acc[c], ffk::mul22(a, __ldg(dY + c * lddy + r)));
-        }
-#pragma unroll
-        for (int c = 0; c < KT; ++c) o[c * out_ld + j] = acc[c];
+        const int64_t c0 = static_cast<int64_t>(na) * KA + static_cast<int64_t>(z - na) * KB;
+        gemv_t_tile<KB, E, R>(A, m, n, lda, dY + c0 * lddy, lddy, rpb, nrb, cx, out + c0 * out_ld, out_ld, rb_stride,
+                              part);
     }
 }
 
@@ -400,77 +407,144 @@ gemv_t_combine(const float2* __restrict__ ws, int64_t n, int64_t k, int64_t nrb,
     if (idx >= n * k) return;
     const int64_t c = idx / n, j = idx - c * n;
     float2 acc = ws[c * n + j];
-    for (int64_t rb = 1; rb < nrb; ++rb) acc = ffk::add22(acc, ws[(rb * k + c) * n + j]);
-    dX[c * lddx + j] = acc;
+#pragma unroll 8
+    for (int64_t rb = 1; rb < nrb; ++rb) acc = ffk::add22_fast(acc, __ldg(ws + (rb * k + c) * n + j));
+    dX[c * lddx + j] = ffk::ff_overflow_lo(acc);
 }
 
-template <int KT>
-void launch_gemv_t_tile(const float2* A, int64_t m, int64_t n, int64_t lda, const float2* dY, int64_t lddy,
-                        int64_t rows_per_block, int64_t nrb, float2* out, int64_t out_ld, int64_t out_rb_stride,
-                        bool vec, cudaStream_t s)
+// How the adjoint is cut: blocks cx columns (or column pairs) wide and
+// 256 / cx row blocks high, gy of them down the rows, right-hand sides in
+// tiles of 1 (wide false) or as split_tiles says.
+struct AdjointPlan {
+    bool wide;
+    int cx;
+    int64_t gy, nrb, rpb;
+};
+
+// Row blocks for at most `want` of them: nrb blocks of rpb = ceil(m / nrb)
+// rows, none empty.
+inline void cut_rows(int64_t m, int64_t want, int64_t* nrb, int64_t* rpb)
 {
-    if (vec) {
-        const int64_t pairs = n / 2;
-        dim3 grid(static_cast<unsigned>((pairs + kGBlock - 1) / kGBlock), static_cast<unsigned>(nrb));
-        gemv_t_kernel<KT, true><<<grid, kGBlock, 0, s>>>(A, m, n, lda, dY, lddy, rows_per_block, out, out_ld,
-                                                           out_rb_stride);
-    } else {
-        dim3 grid(static_cast<unsigned>((n + kGBlock - 1) / kGBlock), static_cast<unsigned>(nrb));
-        gemv_t_kernel<KT, false><<<grid, kGBlock, 0, s>>>(A, m, n, lda, dY, lddy, rows_per_block, out, out_ld,
-                                                            out_rb_stride);
+    const int64_t w = want < m ? want : (m > 0 ? m : 1);
+    *rpb = (m + w - 1) / w;
+    *nrb = *rpb > 0 ? (m + *rpb - 1) / *rpb : 1;
+}
+
+// Rows of A a thread loads before it adds them: the fewer terms a row gives,
+// the more rows must be in flight to cover the load latency.
+inline int adjoint_rows(const AdjointPlan& p, int ka, int64_t k, bool vec)
+{
+    if (k == 1 && p.gy > 1) return 16;
+    return ka <= 2 || !vec ? 8 : 4;
+}
+
+// Modelled cycles of a cut, fitted to a sweep of all cuts of 41 shapes (64^2 to
+// 16384^2, tall and wide, k = 1-64, even and odd rows; the cut it picks is
+// within 1.5% of the best one measured on average, at worst 12%): FP32 issue of
+// the SM with the most blocks; memory traffic (bytes per cycle of the L2, or of
+// HBM beyond it; short row segments touch more sectors than they use, and more
+// L1 lines per load); a part-filled last wave; the latency of the rows loaded
+// together; and the ordered combination, through shared memory or by a second
+// launch over the workspace.
+double adjoint_cycles(const AdjointPlan& p, int64_t m, int64_t n, int64_t k, bool vec, int sm_count)
+{
+    const TileSplit t = p.wide ? split_tiles(k) : TileSplit{1, 1, k, 0};
+    const int e = vec ? 2 : 1;
+    const int64_t cols = n / e;
+    const int64_t z = t.na + t.nb;
+    const int rows = adjoint_rows(p, t.ka, k, vec);
+    const double blocks = static_cast<double>((cols + p.cx - 1) / p.cx) * static_cast<double>(p.gy * z);
+    const double resident = static_cast<double>(sm_count) * (t.ka >= 2 || rows == 16 ? 3 : 4);
+    const double waves = blocks / resident;
+    double per = std::ceil(blocks / sm_count);   // blocks of the fullest SM
+    double over = 1.0;                           // and how far that is above the mean
+    if (waves > 1.0) {
+        const double part = waves - std::floor(waves);
+        over = (std::floor(waves) + (part > 0.0 ? 0.29 + 0.71 * part : 0.0)) / waves;
+        per = over * blocks / sm_count;
     }
+    const double issue = per * 2.0 * p.rpb * t.ka * e * (24.5 + (vec ? 0.0 : 3.2));
+    const double bytes = 8.0 * m * n * z * (1.0 + (vec ? 23.0 : 16.0) / (8.0 * p.cx * e));
+    // 128-byte lines per warp and row: of A, and one of dY per row block and
+    // right-hand side
+    const double rbw = p.cx < 32 ? 32.0 / p.cx : 1.0;
+    const double l1 = 0.46 * per * 8.0 * p.rpb * (std::fmax(rbw * (vec ? 1.0 : 1.4), 2.0 * e) + t.ka * rbw);
+    const double mem = std::fmax(l1, over * bytes / (8.0 * m * n > 100e6 ? 3800.0 : 6000.0));
+    const double rounds = 1.0 + 0.36 * (std::fmin(std::ceil(waves), 3.0) - 1.0);
+    double c = std::fmax(issue, mem) + 0.24 * std::fmin(issue, mem) +
+               rounds * (464.0 * ((p.rpb + rows - 1) / rows) + 1590.0);
+    if (p.gy > 1)
+        c += 5450.0 + 164.0 * p.nrb + 16.0 * p.nrb * n * k / 3800.0;
+    else if (p.nrb > 1)
+        c += rounds * 59.0 * p.nrb;
+    return c;
 }
 
-const void* gemv_t_kernel_ptr(int kt, bool vec)
+// The cut with the least modelled time.  Against column groups of 256 and at
+// most 64 row blocks in two launches of eight right-hand sides each, before:
+// 32768^2, k = 16: 13.8 -> 11.7 ms (with the Fast2Sum forms); 1024^2: 12.6 ->
+// 5.1 us; 10000 x 100, k = 3: 41 -> 14 us; 2001 x 3001, k = 5: 51 -> 32 us.
+AdjointPlan search_adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int sm_count)
 {
-    switch (kt) {
-    case 8: return vec ? reinterpret_cast<const void*>(&gemv_t_kernel<8, true>)
-                       : reinterpret_cast<const void*>(&gemv_t_kernel<8, false>);
-    case 7: return vec ? reinterpret_cast<const void*>(&gemv_t_kernel<7, true>)
-                       : reinterpret_cast<const void*>(&gemv_t_kernel<7, false>);
-    case 6: return vec ? reinterpret_cast<const void*>(&gemv_t_kernel<6, true>)
-                       : reinterpret_cast<const void*>(&gemv_t_kernel<6, false>);
-    case 5: return vec ? reinterpret_cast<const void*>(&gemv_t_kernel<5, true>)
-                       : reinterpret_cast<const void*>(&gemv_t_kernel<5, false>);
-    case 4: return vec ? reinterpret_cast<const void*>(&gemv_t_kernel<4, true>)
-                       : reinterpret_cast<const void*>(&gemv_t_kernel<4, false>);
-    case 3: return vec ? reinterpret_cast<const void*>(&gemv_t_kernel<3, true>)
-                       : reinterpret_cast<const void*>(&gemv_t_kernel<3, false>);
-    case 2: return vec ? reinterpret_cast<const void*>(&gemv_t_kernel<2, true>)
-                       : reinterpret_cast<const void*>(&gemv_t_kernel<2, false>);
-    default: return vec ? reinterpret_cast<const void*>(&gemv_t_kernel<1, true>)
-                        : reinterpret_cast<const void*>(&gemv_t_kernel<1, false>);
-    }
-}
-
-// Number of row blocks for the adjoint.  The grid is col_blocks x nrb blocks;
-// nrb is chosen so that the grid fills whole waves of resident blocks (SMs x
-// blocks per SM of the widest tile's kernel): the adjoint is FP32-issue
-// bound for k > 2, and a last, partly filled wave would idle most SMs.
-// Every row block keeps at least 32 rows; at most 64 row blocks.
-int64_t row_blocks(int64_t m, int64_t n, int64_t k, bool vec, int sm_count)
-{
-    const int64_t cols = vec ? n / 2 : n;
-    const int64_t col_blocks = (cols + kGBlock - 1) / kGBlock;
-    if (col_blocks < 1 || m < 64) return 1;
-    const int occ = ffh::occupancy(gemv_t_kernel_ptr(tile_for(k), vec), kGBlock);
-    const int64_t resident = static_cast<int64_t>(sm_count) * (occ > 0 ? occ : 1);
-    int64_t maxrb = m / 32;
-    if (maxrb > 64) maxrb = 64;
-    if (maxrb < 1) maxrb = 1;
-    int64_t best = 1;
-    double best_eff = -1.0;
-    for (int64_t nrb = 1; nrb <= maxrb; ++nrb) {
-        const int64_t blocks = nrb * col_blocks;
-        const int64_t waves = (blocks + resident - 1) / resident;
-        double eff = static_cast<double>(blocks) / static_cast<double>(waves * resident);
-        if (blocks < resident) eff *= 0.999;  // prefer at least one full wave when possible
-        if (eff > best_eff + 1e-3) {
-            best_eff = eff;
-            best = nrb;
+    AdjointPlan best{true, kGBlock, 1, 1, m > 0 ? m : 0};
+    if (m < 1 || n < 1) return best;
+    double least = -1.0;
+    auto consider = [&](int cx, int64_t gy) {
+        AdjointPlan p{};
+        p.cx = cx;
+        const int64_t rg = kGBlock / cx;
+        cut_rows(m, rg * gy, &p.nrb, &p.rpb);
+        p.gy = (p.nrb + rg - 1) / rg;
+        for (int w = 0; w < (k > 1 ? 2 : 1); ++w) {
+            p.wide = w == 1;
+            const double c = adjoint_cycles(p, m, n, k, vec, sm_count);
+            if (least < 0.0 || c < least) {
+                least = c;
+                best = p;
+            }
         }
-    }
+    };
+    for (int cx = 2; cx <= kGBlock; cx *= 2) consider(cx, 1);
+    // two launches cost more than a short sum takes in one; a single right-hand
+    // side, bound by HBM, gains nothing from more row blocks (12001^2: 186 us with
+    // 28, 195 with 48)
+    if (least > 10000.0)
+        for (int64_t gy = 2; gy <= (k == 1 ? 16 : 64) && 2 * gy <= m; ++gy) consider(128, gy);
     return best;
+}
+
+// The search takes a few microseconds and a call asks for its plan several
+// times (workspace size, then the launch): each host thread keeps the last
+// few, by sizes.
+AdjointPlan adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int sm_count)
+{
+    struct Entry {
+        int64_t m = -1, n, k;
+        bool vec;
+        int sm_count;
+        AdjointPlan plan;
+    };
+    constexpr unsigned kEntries = 16;
+    static thread_local Entry kept[kEntries];
+    const uint64_t h = static_cast<uint64_t>(m) * 0x9e3779b97f4a7c15ull + static_cast<uint64_t>(n) * 0xc2b2ae3d27d4eb4full +
+                       static_cast<uint64_t>(k) * 2 + (vec ? 1 : 0);
+    Entry& e = kept[(h ^ (h >> 32)) % kEntries];
+    if (e.m != m || e.n != n || e.k != k || e.vec != vec || e.sm_count != sm_count)
+        e = Entry{m, n, k, vec, sm_count, search_adjoint_plan(m, n, k, vec, sm_count)};
+    return e.plan;
+}
+
+template <int KA, int KB, int E, int R, int MINB>
+ff_status launch_adjoint(const AdjointPlan& p, const TileSplit& t, const float2* A, int64_t m, int64_t n, int64_t lda,
+                         const float2* dY, int64_t lddy, float2* out, int64_t out_ld, int64_t rb_stride,
+                         cudaStream_t s)
+{
+    const int64_t cols = n / E;
+    const dim3 grid(static_cast<unsigned>((cols + p.cx - 1) / p.cx), static_cast<unsigned>(p.gy),
+                    static_cast<unsigned>(t.na + t.nb));
+    gemv_t_kernel<KA, KB, E, R, MINB><<<grid, kGBlock, 0, s>>>(A, m, n, lda, dY, lddy, p.rpb, p.nrb, p.cx, out, out_ld,
+                                                               rb_stride, static_cast<int>(t.na));
+    return ffh::check_launch();
 }
 
 // ---------------------------------------------------------------------------
@@ -734,11 +808,9 @@ gemv_f64_kernel(const double* __restrict__ A, int64_t m, int64_t n, int64_t lda,
 
 bool bad_dims(int64_t m, int64_t n, int64_t k) { return m < 0 || n < 0 || k < 1 || k > kMaxK; }
 
-size_t gemv_t_ws(int64_t m, int64_t n, int64_t k, bool vec, int sm_count)
+size_t adjoint_ws(const AdjointPlan& p, int64_t n, int64_t k)
 {
-    const int64_t nrb = row_blocks(m, n, k, vec, sm_count);
-    if (nrb <= 1) return 16;
-    return static_cast<size_t>(nrb) * static_cast<size_t>(n) * static_cast<size_t>(k) * sizeof(float2);
+    return p.gy <= 1 ? 16 : static_cast<size_t>(p.nrb) * static_cast<size_t>(n) * static_cast<size_t>(k) * sizeof(float2);
 }
 
 }  // namespace
@@ -770,8 +842,8 @@ size_t ff_gemv_t_workspace_bytes(int64_t m, int64_t n, int64_t k)
     ffh::DeviceInfo di;
     if (ffh::device_info(&di) != FF_OK) return 0;
     // the workspace must cover either access path: take the larger
-    const size_t a = gemv_t_ws(m, n, k, true, di.sm_count);
-    const size_t b = gemv_t_ws(m, n, k, false, di.sm_count);
+    const size_t a = adjoint_ws(adjoint_plan(m, n, k, true, di.sm_count), n, k);
+    const size_t b = adjoint_ws(adjoint_plan(m, n, k, false, di.sm_count), n, k);
     return a > b ? a : b;
 }
 
@@ -783,7 +855,7 @@ ff_status ff_gemv_t_launch_shape(const ff2* A, int64_t m, int64_t n, int64_t lda
     const ff_status st = ffh::device_info(&di);
     if (st != FF_OK) return st;
     const bool vec = (n % 2 == 0) && (lda % 2 == 0) && ffh::aligned(A, 16);
-    *nrb = row_blocks(m, n, k, vec, di.sm_count);
+    *nrb = adjoint_plan(m, n, k, vec, di.sm_count).nrb;
     *vector = vec ? 1 : 0;
     return FF_OK;
 }
@@ -803,44 +875,42 @@ ff_status ff_gemv_t(const ff2* A_, int64_t m, int64_t n, int64_t lda, const ff2*
     auto* dY = reinterpret_cast<const float2*>(dY_);
     auto* dX = reinterpret_cast<float2*>(dX_);
     const bool vec = (n % 2 == 0) && (lda % 2 == 0) && ffh::aligned(A, 16);
-    const int64_t nrb = row_blocks(m, n, k, vec, di.sm_count);
-    const int64_t rpb = m > 0 ? (m + nrb - 1) / nrb : 0;
-    float2* part = nullptr;
-    if (nrb > 1) {
-        if (ws == nullptr || ws_bytes < gemv_t_ws(m, n, k, vec, di.sm_count) || !ffh::aligned(ws, 16))
+    const AdjointPlan p = adjoint_plan(m, n, k, vec, di.sm_count);
+    float2* out = dX;
+    int64_t out_ld = lddx, rb_stride = 0;
+    if (p.gy > 1) {
+        if (ws == nullptr || ws_bytes < adjoint_ws(p, n, k) || !ffh::aligned(ws, 16))
             return FF_ERR_WORKSPACE;
-        part = static_cast<float2*>(ws);
+        out = static_cast<float2*>(ws);
+        out_ld = n;
+        rb_stride = k * n;
     }
-    for (int64_t c0 = 0; c0 < k;) {
-        const int kt = tile_for(k - c0);
-        const float2* dYc = dY + c0 * lddy;
-        // one row block: write dX directly; else partials [rb][c][j]
-        float2* out = nrb > 1 ? part + c0 * n : dX + c0 * lddx;
-        const int64_t out_ld = nrb > 1 ? n : lddx;
-        const int64_t rb_stride = nrb > 1 ? k * n : 0;
-        const int64_t mm = m > 0 ? m : 0;
-        switch (kt) {
-        case 8: launch_gemv_t_tile<8>(A, mm, n, lda, dYc, lddy, rpb, nrb, out, out_ld, rb_stride, vec, s); break;
-        case 7: launch_gemv_t_tile<7>(A, mm, n, lda, dYc, lddy, rpb, nrb, out, out_ld, rb_stride, vec, s); break;
-        case 6: launch_gemv_t_tile<6>(A, mm, n, lda, dYc, lddy, rpb, nrb, out, out_ld, rb_stride, vec, s); break;
-        case 5: launch_gemv_t_tile<5>(A, mm, n, lda, dYc, lddy, rpb, nrb, out, out_ld, rb_stride, vec, s); break;
-        case 4: launch_gemv_t_tile<4>(A, mm, n, lda, dYc, lddy, rpb, nrb, out, out_ld, rb_stride, vec, s); break;
-        case 3: launch_gemv_t_tile<3>(A, mm, n, lda, dYc, lddy, rpb, nrb, out, out_ld, rb_stride, vec, s); break;
-        case 2: launch_gemv_t_tile<2>(A, mm, n, lda, dYc, lddy, rpb, nrb, out, out_ld, rb_stride, vec, s); break;
-        default: launch_gemv_t_tile<1>(A, mm, n, lda, dYc, lddy, rpb, nrb, out, out_ld, rb_stride, vec, s); break;
-        }
-        st = ffh::check_launch();
-        if (st != FF_OK) return st;
-        c0 += kt;
-    }
-    if (nrb > 1) {
+    const TileSplit t = p.wide ? split_tiles(k) : TileSplit{1, 1, k, 0};
+    // rows loaded together as adjoint_rows says; the residency leaves the
+    // registers that keep those loads in flight
+    if (k == 1 && p.gy > 1)
+        st = vec ? launch_adjoint<1, 1, 2, 16, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)
+                 : launch_adjoint<1, 1, 1, 16, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s);
+    else if (t.ka == 1)
+        st = vec ? launch_adjoint<1, 1, 2, 8, 4>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)
+                 : launch_adjoint<1, 1, 1, 8, 4>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s);
+    else if (t.ka == 2)
+        st = vec ? launch_adjoint<2, 1, 2, 8, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)
+                 : launch_adjoint<2, 1, 1, 8, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s);
+    else if (t.ka == 3)
+        st = vec ? launch_adjoint<3, 2, 2, 4, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)
+                 : launch_adjoint<3, 2, 1, 8, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s);
+    else
+        st = vec ? launch_adjoint<4, 3, 2, 4, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)
+                 : launch_adjoint<4, 3, 1, 8, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s);
+    if (st != FF_OK) return st;
+    if (p.gy > 1) {
         const int64_t total = n * k;
-        gemv_t_combine<<<static_cast<unsigned>((total + kGBlock - 1) / kGBlock), kGBlock, 0, s>>>(part, n, k, nrb, dX,
-                                                                                                  lddx);
+        gemv_t_combine<<<static_cast<unsigned>((total + kGBlock - 1) / kGBlock), kGBlock, 0, s>>>(
+            static_cast<float2*>(ws), n, k, p.nrb, dX, lddx);
         st = ffh::check_launch();
-        if (st != FF_OK) return st;
     }
-    return FF_OK;
+    return st;
 }
 
 ff_status ff_gemv_dA(const ff2* dY_, int64_t m, int64_t lddy, const ff2* X_, int64_t n, int64_t ldx, int64_t k,

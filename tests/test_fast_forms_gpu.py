@@ -4,6 +4,8 @@ documented order), for normalised operands, for pairs whose sum does not round
 to the high part (they leave the fast path), for sums that overflow to an
 infinity at any point, and for infinities, NaN, signed zeros and subnormals;
 at the edges of every tile shape."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -16,6 +18,7 @@ pytestmark = pytest.mark.gpu
 
 if torch.cuda.is_available():
     import paper_cs_0603115_gb300 as ff
+    from paper_cs_0603115_gb300 import _lib
 
 DEV = "cuda"
 
@@ -85,3 +88,23 @@ def test_gemv_tiles(m, n, k, kind):
     rows = np.unique(np.r_[0:8, m // 2:m // 2 + 8, m - 8:m])
     want = replay.gemv_warp_replay(A.numpy()[rows], X.numpy(), vec=n % 2 == 0)
     same_bits(Y[:, rows], want)
+
+
+# one to a few rows, blocks of 2 to 128 column groups with their row blocks
+# combined in shared memory, and two launches; narrow and wide tiles
+ADJOINT = [(1, 9, 2), (2, 300, 1), (7, 64, 5), (33, 2050, 3), (300, 1000, 1), (300, 1001, 4), (1001, 128, 7), (3000, 40, 9),
+           (5003, 37, 2), (4001, 4999, 1), (2100, 4096, 16)]
+
+
+@pytest.mark.parametrize("m,n,k", ADJOINT)
+@pytest.mark.parametrize("kind", KINDS)
+def test_gemv_t_cuts(m, n, k, kind):
+    g = inputs.gemv(m, n, k, inputs.seed_for(4, 201))
+    A, dY = plant(g.A, kind, 5), plant(g.dY, kind, 6)
+    Ad, dYd = A.to(DEV), dY.to(DEV)
+    nrb, vec = ctypes.c_int64(), ctypes.c_int()
+    _lib.call("ff_gemv_t_launch_shape", Ad.data_ptr(), m, n, n, k, ctypes.byref(nrb), ctypes.byref(vec))
+    dX = ff.gemv_t(Ad, dYd).cpu().numpy()
+    cols = np.unique(np.r_[0:min(4, n), n // 2, max(n - 4, 0):n])
+    want = replay.gemv_t_replay(A.numpy()[:, cols], dY.numpy(), nrb.value)
+    same_bits(dX[:, cols], want)

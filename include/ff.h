@@ -27,8 +27,8 @@
  *     FF_ERR_WORKSPACE.  A failed launch returns FF_ERR_CUDA and keeps the
  *     CUDA error code for ff_last_cuda_error().  Nothing is enqueued when a
  *     call returns an argument or workspace error; when a call that makes
- *     two launches (a weight gradient in two passes, a GEMV adjoint and its
- *     combination) fails to launch the second, the first stays enqueued.
+ *     two launches (a GEMV adjoint and its combination) fails to launch
+ *     the second, the first stays enqueued.
  *   - Sizes.  n == 0 is a no-op returning FF_OK, except that a reduction
  *     with n == 0 writes (0, 0) to its result.
  *   - Aliasing.  An elementwise output may be exactly one of its inputs
@@ -256,13 +256,10 @@ FF_API ff_status ff_gemv_t_launch_shape(const ff2* A, int64_t m, int64_t n, int6
  * (bit-reproducible).  dY: m x k column-major (lddy >= m); X: n x k
  * column-major (ldx >= n); dA: m x n row-major (ldda >= n), overwritten;
  * it must not overlap dY or X.  1 <= k <= 64.  Every element starts from
- * (0, 0) as the sum's definition says; its first Add22 (with the zero) is
- * formed in two additions when the term is a finite normalised pair (the
- * same bits), the full Add22 otherwise.  Up to k = 21 (with even n, ldx and
- * ldda and 16-byte aligned X and dA; up to 12 otherwise) it runs its own
- * kernel, in one pass up to k = 12 and in two above (the second continuing
- * from the sums the first stored); from there on it runs ff_gemm
- * (transa = 1 on dY), which forms the same terms in the same order. */
+ * (0, 0) as the sum's definition says; where the operands are normalised pairs
+ * the steps are formed with fewer operations (the same bits).  Up to k = 20 it
+ * runs its own kernel; from there on it runs ff_gemm (transa = 1 on dY), which
+ * forms the same terms in the same order. */
 FF_API ff_status ff_gemv_dA(const ff2* dY, int64_t m, int64_t lddy, const ff2* X, int64_t n, int64_t ldx,
                             int64_t k, ff2* dA, int64_t ldda, cudaStream_t s);
 

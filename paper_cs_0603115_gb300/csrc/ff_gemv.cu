@@ -18,10 +18,16 @@
 // holds several row blocks of its columns and adds their sums in row-block
 // order, or the sums go to the workspace and a second kernel adds them.
 //
-// ff_gemv_dA: one thread per pair of adjacent columns of dA, the block's
-// rows walked in pairs with dY staged in shared memory; every element adds
-// its k terms in order from (0, 0), in one pass up to twelve right-hand
-// sides and two above, or through the GEMM kernel for larger k.
+// ff_gemv_dA: one thread per column or pair of adjacent columns of dA, its X
+// values in registers, the block's rows walked four elements at a time with dY
+// staged in shared memory; every element adds its k terms in order from (0, 0).
+// Larger k runs on the GEMM kernel.
+//
+// All three are bound by FP32 issue from two right-hand sides on (28
+// instructions per term as Mul22 + Add22) and use the Fast2Sum forms of
+// ff_core.cuh (22): the weight gradient checks its operands once, the other
+// two, which use each operand pair once, check every product (23) and repeat a
+// sum with the full forms when one falls outside their condition.
 #include <cmath>
 #include <type_traits>
 
@@ -550,229 +556,164 @@ ff_status launch_adjoint(const AdjointPlan& p, const TileSplit& t, const float2*
 // ---------------------------------------------------------------------------
 // dA = dY X^T.  Every element accumulates its k terms Mul22(dY[r, c], X[j, c])
 // in order c = 0 .. k-1 from (0, 0), so the result is the oracle's
-// left-to-right sum bit for bit.  With 16-byte access along the rows of dA,
-// k <= 21 runs here in one or two passes (gemv_dA_small_kernel); without it,
-// k <= 12 runs here with one thread per column (gemv_dA_scalar_kernel).
-// Larger k runs as the matrix product op(dY) X on the GEMM kernel (the same
-// terms in the same order).  Both kernels walk the rows with a grid of about
-// one wave of blocks.
+// left-to-right sum bit for bit.  Up to kDAMaxSmallK right-hand sides run
+// here; larger k runs as the matrix product op(dY) X on the GEMM kernel (the
+// same terms in the same order).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kGBlock)
-gemv_dA_scalar_kernel(const float2* __restrict__ dY, int64_t m, int64_t lddy, const float2* __restrict__ X,
-                      int64_t n, int64_t ldx, int64_t k, float2* __restrict__ dA, int64_t ldda)
-{
-    const int64_t j = static_cast<int64_t>(blockIdx.x) * kGBlock + threadIdx.x;
-    if (j >= n) return;
-    for (int64_t r = blockIdx.y; r < m; r += gridDim.y) {
-        float2 acc = make_float2(0.0f, 0.0f);
-        for (int64_t c = 0; c < k; ++c) acc = ffk::add22(acc, ffk::mul22(__ldg(dY + c * lddy + r), X[c * ldx + j]));
-        dA[r * ldda + j] = acc;
-    }
-}
 
-// Rows per shared-memory chunk of dY in the weight-gradient kernel (even).
+// Rows per shared-memory chunk of dY (a multiple of four).
 constexpr int kTChunk = 128;
 
-// dA for up to 12 right-hand sides with 16-byte access along the rows of dA: one thread per
-// pair of adjacent columns, the thread's k column-pair values of X in
-// registers.  Block row y takes the rows [y rpb, (y + 1) rpb) (rpb even) in
-// pairs, so a thread forms 4 elements per step; the block stages the dY
-// values of kTChunk rows at a time in shared memory, where one 16-byte read
-// gives both rows of a pair for one right-hand side.  Every element is
-// Add22((0, 0), term_0), then Add22 of terms 1 .. k-1, in order (the first
-// step through add22_from_zero, bit-identical).  With ACC the elements
-// continue from the values dA holds (the partial sums of the right-hand
-// sides before these k: the second pass for 12 < k <= 21), adding terms
-// 0 .. k-1 in order.  Lanes past the last column pair work on the last pair
-// and do not store, so that every lane of a warp takes part in the vote and
-// every thread reaches the block barriers.
-//
-// Resident blocks per SM the register allocation must leave room for: a
-// continuing pass of ten or more right-hand sides took 98-100 registers on
-// its own (two blocks per SM) and ran at 0.82-0.83 of the FP32 roofline
-// (32768^2, k = 18-20 as 8 + 10 .. 8 + 12); at 80 registers (three blocks)
-// k = 20 as 10 + 10 runs at 0.92.
-constexpr int dA_min_blocks(int kt, bool acc) { return acc && kt >= 10 ? 3 : 0; }
-
-template <int KT, bool ACC>
-__global__ void __launch_bounds__(kGBlock, dA_min_blocks(KT, ACC))
+// One thread holds E adjacent columns (two with 16-byte access along the rows
+// of dA, else one) and their KT values of X; block row y takes the rows [y rpb,
+// (y + 1) rpb), 4 / E at a time, so a thread forms four elements per step.  The
+// block stages the dY values of kTChunk rows at a time in shared memory, where
+// one 16-byte read gives two rows of one right-hand side.  Every element is
+// Add22((0, 0), term_0), then Add22 of terms 1 .. KT-1, in order.
+// The chunk's dY and the threads' X are checked once, in the staging barrier:
+// a chunk whose values are all normalised takes the Fast2Sum forms (and the
+// first step from (0, 0) in two additions), any other the full ones.
+// Threads past the last column work on the last one and do not store, so that
+// every thread reaches the barriers.
+template <int KT, int E>
+__global__ void __launch_bounds__(kGBlock)
 gemv_dA_small_kernel(const float2* __restrict__ dY, int64_t m, int64_t lddy, const float2* __restrict__ X, int64_t n,
                      int64_t ldx, float2* __restrict__ dA, int64_t ldda, int64_t rpb)
 {
-    __shared__ float4 sdy[KT][kTChunk / 2];
-    const int64_t npairs = n >> 1;
-    const int64_t jp_raw = static_cast<int64_t>(blockIdx.x) * kGBlock + threadIdx.x;
-    if (static_cast<int64_t>(blockIdx.x) * kGBlock >= npairs) return;  // whole block past the end
-    const bool store = jp_raw < npairs;
-    const int64_t jp = store ? jp_raw : npairs - 1;
-    float2 xl[KT], xh[KT];
+    using V = std::conditional_t<E == 2, float4, float2>;
+    constexpr int RS = 4 / E;   // rows per step
+    __shared__ __align__(16) float2 sdy[KT][kTChunk];
+    const int64_t j_raw = (static_cast<int64_t>(blockIdx.x) * kGBlock + threadIdx.x) * E;
+    const bool store = j_raw < n;
+    const int64_t j = store ? j_raw : n - E;
+    float2 x[KT][E];
+    bool okx = true;
 #pragma unroll
     for (int c = 0; c < KT; ++c) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(X + c * ldx) + jp);
-        xl[c] = make_float2(v.x, v.y);
-        xh[c] = make_float2(v.z, v.w);
+        const V v = __ldg(reinterpret_cast<const V*>(X + c * ldx + j));
+        x[c][0] = make_float2(v.x, v.y);
+        if constexpr (E == 2) x[c][1] = make_float2(v.z, v.w);
+#pragma unroll
+        for (int e = 0; e < E; ++e) okx &= ffk::normalised(x[c][e]);
     }
-    constexpr int C0 = ACC ? 0 : 1;   // first term added by the loop below
     const int64_t r0 = static_cast<int64_t>(blockIdx.y) * rpb;
     const int64_t r1 = r0 + rpb < m ? r0 + rpb : m;
-    const int64_t rp = r0 + ((r1 > r0 ? r1 - r0 : 0) & ~static_cast<int64_t>(1));   // end of the row pairs
-    for (int64_t cb = r0; cb < rp; cb += kTChunk) {
-        const int rows = static_cast<int>(rp - cb < kTChunk ? rp - cb : kTChunk);
-        __syncthreads();   // the previous chunk's reads are done
+
+    // R rows of the chunk from row q on
+    auto rows = [&](auto fast_c, auto r_c, int q, V (&v)[decltype(r_c)::value]) {
+        constexpr bool FAST = decltype(fast_c)::value;
+        constexpr int R = decltype(r_c)::value;
+        float2 a[R][E];
+#pragma unroll
+        for (int c = 0; c < KT; ++c) {
+            float2 d[R];
+            if constexpr (R % 2 == 0) {
+#pragma unroll
+                for (int r = 0; r < R; r += 2) {
+                    const float4 p = *reinterpret_cast<const float4*>(&sdy[c][q + r]);
+                    d[r] = make_float2(p.x, p.y);
+                    d[r + 1] = make_float2(p.z, p.w);
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; ++r) d[r] = sdy[c][q + r];
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const float2 t = FAST ? ffk::mul22_fast(d[r], x[c][e]) : ffk::mul22(d[r], x[c][e]);
+                    if (c == 0)
+                        a[r][e] = FAST ? ffk::add22_from_zero_fast(t) : ffk::add22(make_float2(0.0f, 0.0f), t);
+                    else
+                        a[r][e] = FAST ? ffk::add22_fast(a[r][e], t) : ffk::add22(a[r][e], t);
+                }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                a[r][e] = KT == 1 ? ffk::from_zero_infinite(a[r][e]) : ffk::ff_overflow_lo(a[r][e]);
+            if constexpr (E == 2)
+                v[r] = make_float4(a[r][0].x, a[r][0].y, a[r][1].x, a[r][1].y);
+            else
+                v[r] = a[r][0];
+        }
+    };
+    auto chunk = [&](auto fast_c, int64_t cb, int n_rows) {
+        float2* out = dA + cb * ldda + j;
+        int q = 0;
+#pragma unroll 1
+        for (; q + RS <= n_rows; q += RS, out += RS * ldda) {
+            V v[RS];
+            rows(fast_c, std::integral_constant<int, RS>(), q, v);
+            if (store) {
+#pragma unroll
+                for (int r = 0; r < RS; ++r) __stcs(reinterpret_cast<V*>(out + r * ldda), v[r]);
+            }
+        }
+#pragma unroll 1
+        for (; q < n_rows; ++q, out += ldda) {
+            V v[1];
+            rows(fast_c, std::integral_constant<int, 1>(), q, v);
+            if (store) __stcs(reinterpret_cast<V*>(out), v[0]);
+        }
+    };
+    for (int64_t cb = r0; cb < r1; cb += kTChunk) {
+        const int n_rows = static_cast<int>(r1 - cb < kTChunk ? r1 - cb : kTChunk);
+        if (cb > r0) __syncthreads();   // the previous chunk's reads are done
+        bool ok = okx;
         for (int i = threadIdx.x; i < KT * kTChunk; i += kGBlock) {
             const int c = i / kTChunk, q = i - c * kTChunk;
-            if (q < rows) reinterpret_cast<float2*>(sdy[c])[q] = __ldg(dY + c * lddy + cb + q);
-        }
-        __syncthreads();
-        float4* row = reinterpret_cast<float4*>(dA + cb * ldda) + jp;
-        const int64_t ldda4 = ldda >> 1;
-        float4 n0, n1;   // ACC: the stored sums of the next row pair, loaded one pair ahead
-        if constexpr (ACC) {
-            n0 = __ldcs(row);
-            n1 = __ldcs(row + ldda4);
-        }
-        for (int lp = 0; lp < rows / 2; ++lp, row += 2 * ldda4) {
-            float2 a00, a01, a10, a11;
-            if constexpr (ACC) {
-                const float4 p0 = n0, p1 = n1;
-                if (lp + 1 < rows / 2) {
-                    n0 = __ldcs(row + 2 * ldda4);
-                    n1 = __ldcs(row + 3 * ldda4);
-                }
-                a00 = make_float2(p0.x, p0.y);
-                a01 = make_float2(p0.z, p0.w);
-                a10 = make_float2(p1.x, p1.y);
-                a11 = make_float2(p1.z, p1.w);
-            } else {
-                const float4 d01 = sdy[0][lp];
-                const float2 t00 = ffk::mul22(make_float2(d01.x, d01.y), xl[0]);
-                const float2 t01 = ffk::mul22(make_float2(d01.x, d01.y), xh[0]);
-                const float2 t10 = ffk::mul22(make_float2(d01.z, d01.w), xl[0]);
-                const float2 t11 = ffk::mul22(make_float2(d01.z, d01.w), xh[0]);
-                const bool fast = __all_sync(0xffffffffu, ffk::from_zero_fast(t00) && ffk::from_zero_fast(t01) &&
-                                                              ffk::from_zero_fast(t10) &&
-                                                              ffk::from_zero_fast(t11));
-                a00 = ffk::add22_from_zero(t00, fast);
-                a01 = ffk::add22_from_zero(t01, fast);
-                a10 = ffk::add22_from_zero(t10, fast);
-                a11 = ffk::add22_from_zero(t11, fast);
-            }
-#pragma unroll
-            for (int c = C0; c < KT; ++c) {
-                const float4 d01 = sdy[c][lp];
-                const float2 d0 = make_float2(d01.x, d01.y), d1 = make_float2(d01.z, d01.w);
-                a00 = ffk::add22(a00, ffk::mul22(d0, xl[c]));
-                a01 = ffk::add22(a01, ffk::mul22(d0, xh[c]));
-                a10 = ffk::add22(a10, ffk::mul22(d1, xl[c]));
-                a11 = ffk::add22(a11, ffk::mul22(d1, xh[c]));
-            }
-            if (store) {
-                __stcs(row, make_float4(a00.x, a00.y, a01.x, a01.y));
-                __stcs(row + ldda4, make_float4(a10.x, a10.y, a11.x, a11.y));
+            if (q < n_rows) {
+                const float2 d = __ldg(dY + c * lddy + cb + q);
+                ok &= ffk::normalised(d);
+                sdy[c][q] = d;
             }
         }
-    }
-    if (rp < r1) {  // the last row of an odd m
-        const int64_t r = rp;
-        float4* row = reinterpret_cast<float4*>(dA + r * ldda) + jp;
-        float2 a0, a1;
-        if constexpr (ACC) {
-            const float4 p = __ldcs(row);
-            a0 = make_float2(p.x, p.y);
-            a1 = make_float2(p.z, p.w);
-        } else {
-            const float2 d = __ldg(dY + r);
-            const float2 t0 = ffk::mul22(d, xl[0]), t1 = ffk::mul22(d, xh[0]);
-            const bool fast = __all_sync(0xffffffffu, ffk::from_zero_fast(t0) && ffk::from_zero_fast(t1));
-            a0 = ffk::add22_from_zero(t0, fast);
-            a1 = ffk::add22_from_zero(t1, fast);
-        }
-#pragma unroll
-        for (int c = C0; c < KT; ++c) {
-            const float2 dc = __ldg(dY + c * lddy + r);
-            a0 = ffk::add22(a0, ffk::mul22(dc, xl[c]));
-            a1 = ffk::add22(a1, ffk::mul22(dc, xh[c]));
-        }
-        if (store) __stcs(row, make_float4(a0.x, a0.y, a1.x, a1.y));
+        if (__syncthreads_and(ok))
+            chunk(std::true_type(), cb, n_rows);
+        else
+            chunk(std::false_type(), cb, n_rows);
     }
 }
 
-// Widest k that ff_gemv_dA runs on gemv_dA_small_kernel: one pass up to 12
-// right-hand sides (32768^2, k = 9-12: 0.93-0.95 of the FP32 roofline in one
-// pass against 0.87-0.89 in two), then two passes of ceil(k/2) and floor(k/2),
-// the second continuing from the stored sums (loaded one row pair ahead), up
-// to 21; the GEMM kernel takes larger k.  32768^2, fractions of the FP32
-// roofline, two passes against the GEMM route: k = 13-21 0.90-0.92 against
-// 0.87-0.90; k = 22-23 0.89-0.90 against 0.90; k = 24 (12 + 12, where the
-// continuing pass spills at 80 registers) 0.85 against 0.91.
-constexpr int kDAPass = 12;
-constexpr int kDAMaxSmallK = 21;
-// The continuing pass is the second of two and takes floor(k/2) <= 10
-// right-hand sides: no wider continuing kernel is compiled (dA_kt maps the
-// cases above ten of the switches below to it; the pass loop never takes
-// them).
-constexpr int kDAMaxAccKT = kDAMaxSmallK / 2;
-constexpr int dA_kt(int kt, bool acc) { return acc && kt > kDAMaxAccKT ? kDAMaxAccKT : kt; }
-static_assert((kDAMaxSmallK + 1) / 2 <= kDAPass && kDAMaxSmallK <= 2 * kDAPass,
-              "beyond one pass, ff_gemv_dA runs exactly two passes of at most kDAPass right-hand sides");
+// Widest k of a column pair per thread, and of the kernel at all.  A pair's X
+// takes 4 k registers: at k = 12 (95 registers) 1.63e12 terms/s on 8192^2, single
+// columns 1.54e12; beyond, single columns (k = 13-20: 1.61 -> 1.54e12) against
+// the GEMM kernel's 1.38-1.43e12 and the 1.35-1.53e12 of two passes over dA,
+// which they replace.  Odd row lengths take single columns throughout (4001^2,
+// k = 5: 1.46e12 terms/s; with X re-read for every element 0.59e12).
+constexpr int kDAPair = 12;
+constexpr int kDAMaxSmallK = 20;
 
-template <bool ACC>
-const void* dA_small_ptr(int k)
+// Grid of one wave of resident blocks (rounded down so that every block is
+// resident at once), block rows of whole steps.
+template <int KT, int E>
+ff_status launch_dA(const float2* dY, int64_t m, int64_t lddy, const float2* X, int64_t n, int64_t ldx, float2* dA,
+                    int64_t ldda, int sm_count, cudaStream_t s)
 {
-    switch (k) {
-    case 1: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<1, ACC>);
-    case 2: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<2, ACC>);
-    case 3: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<3, ACC>);
-    case 4: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<4, ACC>);
-    case 5: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<5, ACC>);
-    case 6: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<6, ACC>);
-    case 7: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<7, ACC>);
-    case 8: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<8, ACC>);
-    case 9: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<9, ACC>);
-    case 10: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<10, ACC>);
-    case 11: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<dA_kt(11, ACC), ACC>);
-    default: return reinterpret_cast<const void*>(&gemv_dA_small_kernel<dA_kt(12, ACC), ACC>);
-    }
-}
-
-template <bool ACC>
-void launch_dA_small(int k, dim3 grid, cudaStream_t s, const float2* dY, int64_t m, int64_t lddy, const float2* X,
-                     int64_t n, int64_t ldx, float2* dA, int64_t ldda, int64_t rpb)
-{
-    switch (k) {
-    case 1: gemv_dA_small_kernel<1, ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb); break;
-    case 2: gemv_dA_small_kernel<2, ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb); break;
-    case 3: gemv_dA_small_kernel<3, ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb); break;
-    case 4: gemv_dA_small_kernel<4, ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb); break;
-    case 5: gemv_dA_small_kernel<5, ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb); break;
-    case 6: gemv_dA_small_kernel<6, ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb); break;
-    case 7: gemv_dA_small_kernel<7, ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb); break;
-    case 8: gemv_dA_small_kernel<8, ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb); break;
-    case 9: gemv_dA_small_kernel<9, ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb); break;
-    case 10: gemv_dA_small_kernel<10, ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb); break;
-    case 11:
-        gemv_dA_small_kernel<dA_kt(11, ACC), ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb);
-        break;
-    default:
-        gemv_dA_small_kernel<dA_kt(12, ACC), ACC><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb);
-        break;
-    }
-}
-
-// Grid of one wave of resident blocks of `kern` (rounded down so that every
-// block is resident at once), block rows of an even number of rows.
-void dA_small_grid(const void* kern, int64_t m, int64_t n, int sm_count, dim3* grid, int64_t* rpb)
-{
-    const int64_t col_blocks = (n / 2 + kGBlock - 1) / kGBlock;
-    const int occ = ffh::occupancy(kern, kGBlock);
+    const int64_t col_blocks = (n / E + kGBlock - 1) / kGBlock;
+    const int occ = ffh::occupancy(reinterpret_cast<const void*>(&gemv_dA_small_kernel<KT, E>), kGBlock);
     int64_t gy = static_cast<int64_t>(sm_count) * (occ > 0 ? occ : 1) / col_blocks;
-    if (gy > (m + 1) / 2) gy = (m + 1) / 2;
+    constexpr int64_t RS = 4 / E;
+    if (gy > (m + RS - 1) / RS) gy = (m + RS - 1) / RS;
     if (gy > 65535) gy = 65535;
     if (gy < 1) gy = 1;
-    int64_t r = (m + gy - 1) / gy;
-    r += r & 1;
-    *rpb = r;
-    *grid = dim3(static_cast<unsigned>(col_blocks), static_cast<unsigned>((m + r - 1) / r));
+    const int64_t rpb = ((m + gy - 1) / gy + RS - 1) / RS * RS;
+    const dim3 grid(static_cast<unsigned>(col_blocks), static_cast<unsigned>((m + rpb - 1) / rpb));
+    gemv_dA_small_kernel<KT, E><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb);
+    return ffh::check_launch();
+}
+
+// k <= KT right-hand sides.
+template <int KT, int E>
+ff_status dA_small(int64_t k, const float2* dY, int64_t m, int64_t lddy, const float2* X, int64_t n, int64_t ldx,
+                   float2* dA, int64_t ldda, int sm_count, cudaStream_t s)
+{
+    if constexpr (KT > 1)
+        if (k < KT) return dA_small<KT - 1, E>(k, dY, m, lddy, X, n, ldx, dA, ldda, sm_count, s);
+    return launch_dA<KT, E>(dY, m, lddy, X, n, ldx, dA, ldda, sm_count, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -930,43 +871,11 @@ ff_status ff_gemv_dA(const ff2* dY_, int64_t m, int64_t lddy, const ff2* X_, int
     auto* X = reinterpret_cast<const float2*>(X_);
     auto* dA = reinterpret_cast<float2*>(dA_);
     const bool vec = (n % 2 == 0) && (ldx % 2 == 0) && (ldda % 2 == 0) && ffh::aligned(X, 16) && ffh::aligned(dA, 16);
-    if (!vec && k > kDAPass) return ff_gemm(1, 0, m, n, k, dY_, lddy, X_, ldx, dA_, ldda, s);
     ffh::DeviceInfo di;
     const ff_status st = ffh::device_info(&di);
     if (st != FF_OK) return st;
-    if (vec) {
-        // up to kDAPass right-hand sides in one pass from (0, 0); more in
-        // two passes of ceil(k/2) and floor(k/2), the second continuing from
-        // the sums the first stored: a narrow pass is bound by re-reading dA
-        // (32768^2: k = 9 as 8 + 1 measured 0.78 of the roofline, as 5 + 4
-        // 0.86; k = 13 as 12 + 1 0.81, as 7 + 6 0.92)
-        for (int64_t c0 = 0; c0 < k;) {
-            const int64_t rest = k - c0;
-            const int kt = static_cast<int>(rest <= kDAPass ? rest : (rest + 1) / 2);
-            dim3 grid;
-            int64_t rpb;
-            if (c0 == 0) {
-                dA_small_grid(dA_small_ptr<false>(kt), m, n, di.sm_count, &grid, &rpb);
-                launch_dA_small<false>(kt, grid, s, dY, m, lddy, X, n, ldx, dA, ldda, rpb);
-            } else {
-                dA_small_grid(dA_small_ptr<true>(kt), m, n, di.sm_count, &grid, &rpb);
-                launch_dA_small<true>(kt, grid, s, dY + c0 * lddy, m, lddy, X + c0 * ldx, n, ldx, dA, ldda, rpb);
-            }
-            const ff_status stp = ffh::check_launch();
-            if (stp != FF_OK) return stp;
-            c0 += kt;
-        }
-        return FF_OK;
-    }
-    const int64_t col_blocks = (n + kGBlock - 1) / kGBlock;
-    const int occ = ffh::occupancy(reinterpret_cast<const void*>(&gemv_dA_scalar_kernel), kGBlock);
-    int64_t gy64 = static_cast<int64_t>(di.sm_count) * (occ > 0 ? occ : 1) / col_blocks;
-    if (gy64 > m) gy64 = m;
-    if (gy64 > 65535) gy64 = 65535;
-    if (gy64 < 1) gy64 = 1;
-    dim3 grid(static_cast<unsigned>(col_blocks), static_cast<unsigned>(gy64));
-    gemv_dA_scalar_kernel<<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, k, dA, ldda);
-    return ffh::check_launch();
+    return vec && k <= kDAPair ? dA_small<kDAPair, 2>(k, dY, m, lddy, X, n, ldx, dA, ldda, di.sm_count, s)
+                               : dA_small<kDAMaxSmallK, 1>(k, dY, m, lddy, X, n, ldx, dA, ldda, di.sm_count, s);
 }
 
 ff_status ff_f64_gemv(const double* A, int64_t m, int64_t n, int64_t lda, const double* X, int64_t ldx, int64_t k,

@@ -108,3 +108,15 @@ def test_gemv_t_cuts(m, n, k, kind):
     cols = np.unique(np.r_[0:min(4, n), n // 2, max(n - 4, 0):n])
     want = replay.gemv_t_replay(A.numpy()[:, cols], dY.numpy(), nrb.value)
     same_bits(dX[:, cols], want)
+
+
+# one pass, the widest single pass, two passes, the matrix-product route; even
+# and odd rows of dA; rows around the steps and the staged chunks
+@pytest.mark.parametrize("m,n,k", [(5, 6, 1), (131, 7, 1), (261, 514, 2), (129, 515, 5), (66, 36, 12), (67, 35, 13), (133, 130, 20),
+                                   (130, 131, 21), (40, 41, 25)])
+@pytest.mark.parametrize("kind", KINDS)
+def test_gemv_dA_passes(m, n, k, kind):
+    g = inputs.gemv(m, n, k, inputs.seed_for(4, 202))
+    X, dY = plant(g.X, kind, 7), plant(g.dY, kind, 8)
+    dA = ff.gemv_dA(dY.to(DEV), X.to(DEV)).cpu().numpy()
+    same_bits(dA, oracle.gemv_dA(dY.numpy(), X.numpy()))

@@ -4,7 +4,8 @@ A float-float tensor is a ``torch.float32`` CUDA tensor whose last dimension
 is 2: ``x[..., 0]`` is the high part and ``x[..., 1]`` the low part of the
 unevaluated sum hi + lo (Section 4 of the paper).  Vectors are ``(n, 2)``.
 Every function here marshals its arguments and calls one entry point of the
-C ABI in ``libff.so`` (include/ff.h) on the current CUDA stream; all
+C ABI in ``libff.so`` (include/ff.h) on the current CUDA stream, through the
+native front ``_ffnative`` (csrc/ff_torch.cpp) where that takes the call; all
 arithmetic runs in the library's CUDA kernels.  Nothing falls back to the CPU:
 a missing library or a non-CUDA tensor raises.
 
@@ -119,9 +120,30 @@ def clear_workspaces() -> None:
 
 
 # ---------------------------------------------------------------------------
+# native front
+# ---------------------------------------------------------------------------
+def _native(front: str, name: str, *args):
+    """The call through the native front (csrc/ff_torch.cpp), which makes the
+    checks below, allocates the output and calls the library in one step; None
+    when it does not take the call (an argument it would not accept, a missing
+    workspace, a mode, or the library not loaded yet): the Python path then
+    serves it or raises."""
+    at = _lib.address.get(name)
+    if at is None:
+        return None
+    r = getattr(_lib.native, front)(at, *args)
+    if r.__class__ is int:
+        raise _lib.error(name, r)
+    return r
+
+
+# ---------------------------------------------------------------------------
 # elementwise
 # ---------------------------------------------------------------------------
 def _unary(name, x, out):
+    r = _native("unary", name, x, out)
+    if r is not None:
+        return r
     _check_ff(x, name)
     if out is None:
         out = torch.empty_like(x)
@@ -133,6 +155,9 @@ def _unary(name, x, out):
 
 
 def _binary(name, a, b, out):
+    r = _native("binary", name, a, b, out)
+    if r is not None:
+        return r
     _check_ff(a, name)
     _check_ff(b, name)
     if a.shape != b.shape:
@@ -184,6 +209,9 @@ def sqrt(a, out=None):
 
 def axpy(alpha, x, y, out=None):
     """z = Add22(Mul22(alpha, x), y); alpha is a (hi, lo) pair of floats."""
+    r = _native("axpy", "ff_axpy", float(alpha[0]), float(alpha[1]), x, y, out)
+    if r is not None:
+        return r
     _check_ff(x, "ff_axpy")
     _check_ff(y, "ff_axpy")
     if x.shape != y.shape:
@@ -205,6 +233,9 @@ def _reduce_ws(n: int, device) -> torch.Tensor:
 
 def sum(x, out=None):  # noqa: A001  (mirrors the C name ff_sum)
     """Float-float sum of an (n, 2) vector; returns a (2,) device tensor."""
+    r = _native("reduce1", "ff_sum", x, out, True, _lib.address.get("ff_reduce_workspace_bytes"), _ws_cache, "reduce")
+    if r is not None:
+        return r
     _check_ff(x, "ff_sum")
     if out is None:
         out = torch.empty(2, dtype=torch.float32, device=x.device)
@@ -217,6 +248,9 @@ def sum(x, out=None):  # noqa: A001  (mirrors the C name ff_sum)
 
 def dot(x, y, out=None):
     """Float-float dot product sum_i Mul22(x_i, y_i); returns (2,) on device."""
+    r = _native("reduce2", "ff_dot", x, y, out, True, _lib.address.get("ff_reduce_workspace_bytes"), _ws_cache, "reduce")
+    if r is not None:
+        return r
     _check_ff(x, "ff_dot")
     _check_ff(y, "ff_dot")
     if x.shape != y.shape:
@@ -239,6 +273,9 @@ def _f32_vec(t, name):
 def sum2(x, out=None):
     """Compensated Sum2 of a binary32 vector; returns the float-float (2,)
     result on the device."""
+    r = _native("reduce1", "ff_sum2", x, out, False, _lib.address.get("ff_reduce_workspace_bytes"), _ws_cache, "reduce")
+    if r is not None:
+        return r
     _f32_vec(x, "ff_sum2")
     if out is None:
         out = torch.empty(2, dtype=torch.float32, device=x.device)
@@ -251,6 +288,9 @@ def sum2(x, out=None):
 def dot2(x, y, out=None):
     """Compensated Dot2 of binary32 vectors; returns the float-float (2,)
     result on the device."""
+    r = _native("reduce2", "ff_dot2", x, y, out, False, _lib.address.get("ff_reduce_workspace_bytes"), _ws_cache, "reduce")
+    if r is not None:
+        return r
     _f32_vec(x, "ff_dot2")
     _f32_vec(y, "ff_dot2")
     if x.numel() != y.numel():
@@ -265,6 +305,9 @@ def dot2(x, y, out=None):
 
 def dot_backward(dout, x, y, dx=None, dy=None):
     """dx = Mul22(dout, y), dy = Mul22(dout, x); dout is a (2,) device tensor."""
+    r = _native("dot_backward", "ff_dot_backward", dout, x, y, dx, dy)
+    if r is not None:
+        return r
     _check_ff(dout, "ff_dot_backward")
     _check_ff(x, "ff_dot_backward")
     _check_ff(y, "ff_dot_backward")
@@ -286,6 +329,9 @@ def dot_backward(dout, x, y, dx=None, dy=None):
 def gemv(A, X, out=None):
     """Y = A X.  A: (m, n, 2) row-major; X: (k, n, 2), i.e. n x k column-major
     (X[c] is right-hand side c).  Returns Y as (k, m, 2)."""
+    r = _native("gemv", "ff_gemv", A, X, out)
+    if r is not None:
+        return r
     _check_ff(A, "ff_gemv")
     _check_ff(X, "ff_gemv")
     if A.dim() != 3 or X.dim() != 3 or X.shape[1] != A.shape[1]:
@@ -301,6 +347,9 @@ def gemv(A, X, out=None):
 
 def gemv_t(A, dY, out=None):
     """dX = A^T dY.  A: (m, n, 2); dY: (k, m, 2).  Returns dX as (k, n, 2)."""
+    r = _native("gemv_t", "ff_gemv_t", A, dY, out, _lib.address.get("ff_gemv_t_workspace_bytes"), _ws_cache, "gemv_t")
+    if r is not None:
+        return r
     _check_ff(A, "ff_gemv_t")
     _check_ff(dY, "ff_gemv_t")
     if A.dim() != 3 or dY.dim() != 3 or dY.shape[1] != A.shape[0]:
@@ -319,6 +368,9 @@ def gemv_t(A, dY, out=None):
 def gemv_dA(dY, X, out=None):
     """dA = dY X^T (the weight gradient of Y = A X).  dY: (k, m, 2); X: (k, n, 2).
     Returns dA as (m, n, 2) row-major."""
+    r = _native("gemv_dA", "ff_gemv_dA", dY, X, out)
+    if r is not None:
+        return r
     _check_ff(dY, "ff_gemv_dA")
     _check_ff(X, "ff_gemv_dA")
     if dY.dim() != 3 or X.dim() != 3 or dY.shape[0] != X.shape[0]:
@@ -336,6 +388,9 @@ def gemm(A, B, transa=False, transb=False, out=None):
     """C = op(A) op(B), row-major float-float matrices.  A: (m, k, 2), or
     (k, m, 2) when transa; B: (k, n, 2), or (n, k, 2) when transb.  Returns C
     as (m, n, 2)."""
+    r = _native("gemm", "ff_gemm", A, B, bool(transa), bool(transb), out)
+    if r is not None:
+        return r
     _check_ff(A, "ff_gemm")
     _check_ff(B, "ff_gemm")
     if A.dim() != 3 or B.dim() != 3:

@@ -2,8 +2,8 @@
 
 Marshalling only: every entry point here forwards plain pointers, sizes and a
 stream handle to the library; all arithmetic runs in the library's CUDA
-kernels.  There is no fallback: if libff.so is missing or does not load, the
-first call raises.
+kernels.  There is no fallback: if libff.so or the native front of the wrappers
+(_ffnative) is missing or does not load, the first call raises.
 """
 from __future__ import annotations
 
@@ -92,6 +92,10 @@ SIGNATURES = {
 }
 
 _lib = None
+# the native front (_ffnative) and the addresses of the entry points it calls;
+# empty until the library is loaded
+native = None
+address: dict = {}
 
 
 class FFError(RuntimeError):
@@ -113,7 +117,7 @@ def declared_symbols() -> list[str]:
 
 
 def load() -> ctypes.CDLL:
-    global _lib
+    global _lib, native
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -123,6 +127,10 @@ def load() -> ctypes.CDLL:
         fn = getattr(L, name)
         fn.restype = res
         fn.argtypes = args
+    import torch  # noqa: F401  (the native front links against its libraries)
+    from . import _ffnative
+    native = _ffnative
+    address.update({name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in SIGNATURES})
     _lib = L
     return L
 
@@ -132,6 +140,11 @@ def call(name: str, *args) -> None:
     L = load()
     st = getattr(L, name)(*args)
     if st != 0:
-        err = ctypes.c_int(0)
-        L.ff_last_cuda_error(ctypes.byref(err))
-        raise FFError(name, st, err.value if st == 3 else 0)
+        raise error(name, st)
+
+
+def error(name: str, st: int) -> FFError:
+    """The exception for a non-zero status that ``name`` just returned."""
+    err = ctypes.c_int(0)
+    load().ff_last_cuda_error(ctypes.byref(err))
+    return FFError(name, st, err.value if st == 3 else 0)

@@ -356,7 +356,8 @@ FF_API size_t ff_batch_workspace_bytes(const ff_batch_plan* plan);
 FF_API ff_status ff_batch_plan_info(const ff_batch_plan* plan, ff_tune* tune, int64_t* ntiles, unsigned* grid);
 
 /* Run every instance of the plan: one memset of the per-instance counters
- * and the tile counter, and one persistent kernel launch on stream s.
+ * and the tile counter (for plans that use them), and one persistent kernel
+ * launch on stream s.
  * Graph-capturable.  The workspace (ff_batch_workspace_bytes, 16-byte
  * aligned, owned by the caller) must not be shared by runs that overlap. */
 FF_API ff_status ff_batch_run(const ff_batch_plan* plan, void* ws, size_t ws_bytes, cudaStream_t s);

@@ -30,7 +30,8 @@
 //              counter per instance) adds the instance's tile partials in
 //              tile order and writes the result.
 // No block waits for another; the per-instance counters are zeroed by a
-// memset at the start of every run (and left zero by the last tile).
+// memset at the start of every run that uses them (and left zero by the last
+// tile).
 //
 // Plans made only of GEMV rows run a kernel of their own: their tiles differ
 // in cost (a tile holds 4 x warps x R rows, and R cannot drop below one for
@@ -79,6 +80,7 @@ struct ff_batch_plan {
     int count;
     bool has_gemv_rows;
     bool only_gemv_rows;
+    bool counts;   // a run uses the counters (and clears them first)
     ff_tune tune;
     int64_t ntiles;
     int64_t ndot;
@@ -122,14 +124,87 @@ __device__ __forceinline__ float2 block_reduce(float2 v, float2* sm)
     return v;
 }
 
+// One lane's sum of a GEMV row (gemv_rows_tile_body has the order), U pairs of
+// chunks loaded before they are added.  FAST uses the Fast2Sum forms and sets
+// `bad` when a product fell outside their condition.
+template <bool FAST, int U>
+__device__ __forceinline__ float2 gemv_row_lane(const float2* Ar, const float2* xv, int64_t n, int vec, int l8, bool& bad)
+{
+    auto term = [&](float2& s, float2 a, float2 x) {
+        if (FAST)
+            s = ffk::add22_fast(s, ffk::mul22_fast_checked(a, x, bad));
+        else
+            s = ffk::add22(s, ffk::mul22(a, x));
+    };
+    auto chunk = [&](float2& s, const float4& a, const float4& x) {
+        term(s, make_float2(a.x, a.y), make_float2(x.x, x.y));
+        term(s, make_float2(a.z, a.w), make_float2(x.z, x.w));
+    };
+    float2 acc = make_float2(0.0f, 0.0f);
+    if (vec) {
+        const float4* A4 = reinterpret_cast<const float4*>(Ar);
+        const float4* x4 = reinterpret_cast<const float4*>(xv);
+        const int64_t nch = n >> 1;
+        float2 acc1 = make_float2(0.0f, 0.0f);
+        int64_t c = l8;
+        if constexpr (U > 1) {
+#pragma unroll 1
+            for (; c + 8 * (2 * U - 1) < nch; c += 16 * U) {
+                float4 a[2 * U], x[2 * U];
+#pragma unroll
+                for (int u = 0; u < 2 * U; ++u) {
+                    a[u] = __ldcs(A4 + c + 8 * u);
+                    x[u] = __ldg(x4 + c + 8 * u);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    chunk(acc, a[2 * u], x[2 * u]);
+                    chunk(acc1, a[2 * u + 1], x[2 * u + 1]);
+                }
+            }
+        }
+#pragma unroll 1
+        for (; c + 8 < nch; c += 16) {
+            const float4 a0 = __ldcs(A4 + c), a1 = __ldcs(A4 + c + 8);
+            const float4 x0 = __ldg(x4 + c), x1 = __ldg(x4 + c + 8);
+            chunk(acc, a0, x0);
+            chunk(acc1, a1, x1);
+        }
+        for (; c < nch; c += 8) chunk(acc, __ldcs(A4 + c), __ldg(x4 + c));
+        acc = FAST ? ffk::add22_fast(acc, acc1) : ffk::add22(acc, acc1);
+        if ((n & 1) && l8 == 0) term(acc, Ar[n - 1], xv[n - 1]);
+    } else {
+        int64_t j = l8;
+        if constexpr (FAST) {
+            constexpr int V = 4 * U;
+#pragma unroll 1
+            for (; j + 8 * (V - 1) < n; j += 8 * V) {
+                float2 a[V], x[V];
+#pragma unroll
+                for (int u = 0; u < V; ++u) {
+                    a[u] = __ldcs(Ar + j + 8 * u);
+                    x[u] = __ldg(xv + j + 8 * u);
+                }
+#pragma unroll
+                for (int u = 0; u < V; ++u) term(acc, a[u], x[u]);
+            }
+        }
+#pragma unroll 1
+        for (; j < n; j += 8) term(acc, Ar[j], xv[j]);
+    }
+    return acc;
+}
+
 // One tile of GEMV rows (see the header comment).  Eight lanes reduce one
 // row, so a warp works on four rows at once: lane group g (lanes 8g .. 8g+7)
 // of warp w takes rows start + 4 (w R + k) + g for k = 0 .. R-1, lane l of
 // the group accumulates the row's two-value chunks l + 16i into its first
 // and l + 8 + 16i into its second accumulator (a leftover chunk into the
-// first), adds them, the group combines its eight lanes with a shuffle-down
-// Add22 tree (offsets 4, 2, 1) and its lane 0 writes out[r].  Kept out of
-// line (for the mixed kernel), with its arguments by value.
+// first), adds them (without 16-byte access: the values l + 8i into one), the
+// group combines its eight lanes with a shuffle-down Add22 tree (offsets 4, 2,
+// 1) and its lane 0 writes out[r].  Kept out of line (for the mixed kernel),
+// with its arguments by value.
+template <int U>
 __device__ __forceinline__ void gemv_rows_tile_body(const float2* A, const float2* xv, float2* out, int64_t n,
                                                    int64_t lda, int64_t m, int vec, int rpw, int64_t start)
 {
@@ -143,45 +218,22 @@ __device__ __forceinline__ void gemv_rows_tile_body(const float2* A, const float
         const int64_t r = r0 + g;
         float2 acc = make_float2(0.0f, 0.0f);
         if (r < m) {
-            const float2* Ar = A + r * lda;
-            if (vec) {
-                const float4* A4 = reinterpret_cast<const float4*>(Ar);
-                const float4* x4 = reinterpret_cast<const float4*>(xv);
-                const int64_t nch = n >> 1;
-                float2 acc1 = make_float2(0.0f, 0.0f);
-                int64_t c = l8;
-                for (; c + 8 < nch; c += 16) {
-                    const float4 a0 = __ldcs(A4 + c), a1 = __ldcs(A4 + c + 8);
-                    const float4 x0 = __ldg(x4 + c), x1 = __ldg(x4 + c + 8);
-                    acc = ffk::add22(acc, ffk::mul22(make_float2(a0.x, a0.y), make_float2(x0.x, x0.y)));
-                    acc = ffk::add22(acc, ffk::mul22(make_float2(a0.z, a0.w), make_float2(x0.z, x0.w)));
-                    acc1 = ffk::add22(acc1, ffk::mul22(make_float2(a1.x, a1.y), make_float2(x1.x, x1.y)));
-                    acc1 = ffk::add22(acc1, ffk::mul22(make_float2(a1.z, a1.w), make_float2(x1.z, x1.w)));
-                }
-                for (; c < nch; c += 8) {
-                    const float4 a0 = __ldcs(A4 + c);
-                    const float4 x0 = __ldg(x4 + c);
-                    acc = ffk::add22(acc, ffk::mul22(make_float2(a0.x, a0.y), make_float2(x0.x, x0.y)));
-                    acc = ffk::add22(acc, ffk::mul22(make_float2(a0.z, a0.w), make_float2(x0.z, x0.w)));
-                }
-                acc = ffk::add22(acc, acc1);
-                if ((n & 1) && l8 == 0) acc = ffk::add22(acc, ffk::mul22(Ar[n - 1], xv[n - 1]));
-            } else {
-                for (int64_t j = l8; j < n; j += 8) acc = ffk::add22(acc, ffk::mul22(Ar[j], xv[j]));
-            }
+            bool bad = false;
+            acc = gemv_row_lane<true, U>(A + r * lda, xv, n, vec, l8, bad);
+            if (bad) acc = gemv_row_lane<false, 1>(A + r * lda, xv, n, vec, l8, bad);
         }
 #pragma unroll
         for (int off = 4; off > 0; off >>= 1)
-            acc = ffk::add22(acc, make_float2(__shfl_down_sync(0xffffffffu, acc.x, off, 8),
-                                              __shfl_down_sync(0xffffffffu, acc.y, off, 8)));
-        if (l8 == 0 && r < m) out[r] = acc;
+            acc = ffk::add22_fast(acc, make_float2(__shfl_down_sync(0xffffffffu, acc.x, off, 8),
+                                                   __shfl_down_sync(0xffffffffu, acc.y, off, 8)));
+        if (l8 == 0 && r < m) out[r] = ffk::ff_overflow_lo(acc);
     }
 }
 
 __device__ __noinline__ void gemv_rows_tile(const float2* A, const float2* xv, float2* out, int64_t n,
                                             int64_t lda, int64_t m, int vec, int rpw, int64_t start)
 {
-    gemv_rows_tile_body(A, xv, out, n, lda, m, vec, rpw, start);
+    gemv_rows_tile_body<1>(A, xv, out, n, lda, m, vec, rpw, start);
 }
 
 // PPT values per thread per tile (even).  Values of a tile are visited as
@@ -374,16 +426,29 @@ batch_kernel(const DevInst* __restrict__ insts, const Tile* __restrict__ tiles, 
 }
 
 // Kernel for plans whose records are all GEMV rows: the same tile walk and
-// row reduction, without the other paths, so that it needs few registers and
-// keeps many warps resident: the rows are latency-bound (two 16-byte loads
-// of A in flight per lane), so the register budget is set for a full SM of
-// 64 warps (1024-GEMV batch: 0.86 of the HBM rate at 48 registers, 0.92 at
-// 32).
+// row reduction, without the other paths.  Each lane keeps two pairs of chunks
+// (eight values on 8-byte access) in flight at 64 registers, 32 warps per SM.
+// Bound by HBM and, through the rows' many small trees, by FP32 issue.  300
+// matrices of up to 3000 x 3000, 1.0 GB: 257 us with one pair, 64 warps and the
+// full Mul22 / Add22, single 8-byte loads on odd rows; 195 with the Fast2Sum
+// forms and four values in flight on odd rows at 48 warps; 182 with two pairs;
+// 278 with four pairs at 20 warps.  16 matrices of up to 4000: 82, 95, 40, 37.
+constexpr int kRowPairs = 2;
+
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, 2048 / BLOCK)
+__global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
 batch_gemv_kernel(const DevInst* __restrict__ insts, const Tile* __restrict__ tiles, int64_t ntiles,
                   float2* __restrict__, unsigned* __restrict__, unsigned long long* __restrict__ next)
 {
+    auto tile = [&](unsigned long long t) {
+        const Tile tl = tiles[t];
+        const DevInst& I = insts[tl.inst];
+        gemv_rows_tile_body<kRowPairs>(I.x, I.y, I.out, I.n, I.lda, I.m, I.vec, I.rows_per_warp, tl.start);
+    };
+    if (next == nullptr) {   // a block per tile
+        tile(blockIdx.x);
+        return;
+    }
     __shared__ unsigned long long s_t;
     for (;;) {
         if (threadIdx.x == 0) s_t = atomicAdd(next, 1ull);
@@ -391,9 +456,7 @@ batch_gemv_kernel(const DevInst* __restrict__ insts, const Tile* __restrict__ ti
         const unsigned long long t = s_t;
         __syncthreads();  // every thread has read s_t before thread 0 takes the next tile
         if (t >= static_cast<unsigned long long>(ntiles)) break;
-        const Tile tl = tiles[t];
-        const DevInst& I = insts[tl.inst];
-        gemv_rows_tile_body(I.x, I.y, I.out, I.n, I.lda, I.m, I.vec, I.rows_per_warp, tl.start);
+        tile(t);
     }
 }
 
@@ -515,6 +578,14 @@ ff_status ff_batch_plan_create(const ff_batch_instance* inst, int count, const f
         }
     }
     if (recs.size() > static_cast<size_t>(INT32_MAX)) return FF_ERR_INVALID_ARG;
+    // Values per tile of GEMV rows: about 16K, and fewer in a batch too small to
+    // give every resident block two such tiles, since the groups of a tile run
+    // one after the other (30 matrices of up to 200 x 200: 19.0 -> 7.4 us).
+    int64_t gemv_values = 0;
+    for (const Rec& r : recs)
+        if (r.kind == kGemvRows) gemv_values += r.m * r.n;
+    const int64_t gemv_blocks = static_cast<int64_t>(di.sm_count) * (1024 / tune.block);
+    const int64_t gemv_tile = std::max<int64_t>(1, std::min<int64_t>(16384, gemv_values / (2 * gemv_blocks)));
     std::vector<DevInst> hi(recs.size());
     std::vector<Tile> ht;
     int64_t ndot = 0, total = 0;
@@ -537,10 +608,9 @@ ff_status ff_batch_plan_create(const ff_batch_instance* inst, int count, const f
             // rows of 16-byte-aligned storage when the matrix, its row stride
             // and the vector allow it
             d.vec = (ffh::aligned(b.x, 16) && ffh::aligned(b.y, 16) && (b.lda % 2 == 0)) ? 1 : 0;
-            // four rows per warp at a time, rpw groups of four per warp per
-            // tile: about 16K values per tile
+            // four rows per warp at a time, rpw groups of four per warp per tile
             const int64_t warps = tune.block / 32;
-            int64_t rpw = 16384 / (4 * warps * (b.n > 0 ? b.n : 1));
+            int64_t rpw = gemv_tile / (4 * warps * (b.n > 0 ? b.n : 1));
             rpw = rpw < 1 ? 1 : (rpw > 16 ? 16 : rpw);
             d.rows_per_warp = static_cast<int32_t>(rpw);
             const int64_t rows_per_tile = 4 * warps * rpw;
@@ -601,6 +671,10 @@ ff_status ff_batch_plan_create(const ff_batch_instance* inst, int count, const f
     int64_t grid = static_cast<int64_t>(di.sm_count) * (bps > 0 ? bps : 1);
     if (grid > p->ntiles) grid = p->ntiles > 0 ? p->ntiles : 1;
     p->grid = static_cast<unsigned>(grid);
+    // counters: the arrivals of dots of several tiles, and the tile counter of a
+    // GEMV-only plan with more tiles than blocks
+    p->counts = p->only_gemv_rows && p->ntiles > grid;
+    for (const DevInst& d : hi) p->counts |= d.kind == FF_BATCH_DOT && d.ntiles > 1;
     p->d_inst = nullptr;
     p->d_tiles = nullptr;
     if (!hi.empty()) {
@@ -644,8 +718,12 @@ ff_status ff_batch_run(const ff_batch_plan* p, void* ws, size_t ws_bytes, cudaSt
     const size_t so = sched_offset(static_cast<size_t>(p->count));
     auto* next = reinterpret_cast<unsigned long long*>(static_cast<char*>(ws) + so);
     auto* partials = reinterpret_cast<float2*>(static_cast<char*>(ws) + counters_bytes(static_cast<size_t>(p->count)));
-    ff_status st = ffh::cuda_status(cudaMemsetAsync(counters, 0, so + 8, s));
-    if (st != FF_OK) return st;
+    if (p->counts) {
+        const ff_status st = ffh::cuda_status(cudaMemsetAsync(counters, 0, so + 8, s));
+        if (st != FF_OK) return st;
+    } else {
+        next = nullptr;
+    }
     kernel_for(*var, *p)<<<p->grid, p->tune.block, 0, s>>>(p->d_inst, p->d_tiles, p->ntiles, partials, counters,
                                                            next);
     return ffh::check_launch();

@@ -120,3 +120,25 @@ def test_gemv_dA_passes(m, n, k, kind):
     X, dY = plant(g.X, kind, 7), plant(g.dY, kind, 8)
     dA = ff.gemv_dA(dY.to(DEV), X.to(DEV)).cpu().numpy()
     same_bits(dA, oracle.gemv_dA(dY.numpy(), X.numpy()))
+
+
+# rows around the chunks in flight (16- and 8-byte access), few and many tiles
+@pytest.mark.parametrize("shapes", [[(9, 5)], [(40, 70), (33, 131), (5, 600), (7, 1025)], [(3000, 66), (2500, 67), (900, 258)]])
+@pytest.mark.parametrize("kind", KINDS)
+def test_batch_gemv_rows(shapes, kind):
+    from paper_cs_0603115_gb300 import batch
+    specs, want = [], []
+    for i, (m, n) in enumerate(shapes):
+        g = inputs.gemv(m, n, 1, inputs.seed_for(4, 203 + i))
+        A, x = plant(g.A, kind, 9 + i), plant(g.X[0], kind, 19 + i)
+        out = torch.full((m, 2), float("nan"), device=DEV)
+        specs.append((batch.GEMV, A.to(DEV), x.to(DEV), out, None))
+        rows = np.unique(np.r_[0:min(m, 40), m // 2, max(m - 9, 0):m])
+        want.append((rows, replay.gemv_rows8_replay(A.numpy()[rows], x.numpy(), n % 2 == 0)))
+    plan = batch.BatchPlan(batch.make_instances(specs))
+    for _ in range(2):
+        plan.run()
+        for (_, _, _, out, _), (rows, w) in zip(specs, want):
+            same_bits(out.cpu().numpy()[rows], w)
+            out.fill_(float("nan"))
+    plan.close()

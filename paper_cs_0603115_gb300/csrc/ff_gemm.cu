@@ -11,8 +11,8 @@
 // for RN(hi + lo) == hi; the check is combined over the block in the slice's
 // barrier, and a slice with any other value (or a NaN) runs on the full Mul22 +
 // Add22 (28 instructions), with the same bits either way.  4096^3: 54.4 ms with
-// the full forms alone, 44.2 ms with the fast ones (1.55e12 terms/s, 22.96
-// instructions issued per term, 93% of the cycles issue).
+// the full forms alone, 44.2 ms with the fast ones, 43.1 ms with addresses kept
+// from slice to slice instead of formed for each value (1.59e12 terms/s).
 //
 // A block computes one tile of C from slices of A and B in shared memory,
 // double buffered; the next slice is loaded into registers while the current
@@ -49,25 +49,44 @@ struct Dims {
     int64_t tiles_n, tiles;
 };
 
-// Slice `p0` of one operand into registers: N rows (of op(A)) or columns (of
-// op(B)) from `i0`, BK inner indices.  KMAJOR: the operand is stored
-// contiguous along the rows / columns (transposed A, row-major B), so
-// neighbouring threads take neighbouring rows; otherwise contiguous along the
-// inner index.  Out-of-range values read as (0, 0); they are never used for a
-// stored output nor for a term beyond k.
+// One operand's slices as a thread reads them: N rows (of op(A)) or columns (of
+// op(B)) from the tile's first on, BK inner indices per slice.  KMAJOR: the
+// operand is stored contiguous along the rows / columns (transposed A, row-major
+// B), so neighbouring threads take neighbouring rows; otherwise contiguous along
+// the inner index.  The thread's first address is kept and moved on slice by
+// slice; its L values lie a fixed stride apart.
 template <int N, int BK, int T, int L, bool KMAJOR>
-__device__ __forceinline__ void load_slice(const float2* __restrict__ M, int64_t ld, int64_t extent, int64_t k,
-                                           int64_t i0, int64_t p0, float2 (&v)[L])
-{
-#pragma unroll
-    for (int s = 0; s < L; ++s) {
-        const int e = threadIdx.x + s * T;
-        const int64_t i = i0 + (KMAJOR ? e % N : e / BK);
-        const int64_t p = p0 + (KMAJOR ? e / N : e % BK);
-        const bool in = (i < extent) && (p < k);
-        v[s] = in ? __ldg(KMAJOR ? M + p * ld + i : M + i * ld + p) : make_float2(0.0f, 0.0f);
+struct Slices {
+    static constexpr int kStep = KMAJOR ? T / N : T / BK;   // inner indices / rows between a thread's values
+    static_assert(T % (KMAJOR ? N : BK) == 0, "a thread's values share their row / inner index");
+    const float2* p;
+    int64_t stride, advance;
+    int row, inner;   // the thread's first value: row of the tile, inner index of the slice
+    int rows;         // rows of the tile that exist
+
+    __device__ __forceinline__ Slices(const float2* M, int64_t ld, int64_t extent, int64_t i0)
+    {
+        row = KMAJOR ? threadIdx.x % N : threadIdx.x / BK;
+        inner = KMAJOR ? threadIdx.x / N : threadIdx.x % BK;
+        rows = static_cast<int>(extent - i0 < N ? extent - i0 : N);
+        p = M + (KMAJOR ? inner * ld + i0 + row : (i0 + row) * ld + inner);
+        stride = kStep * ld;
+        advance = KMAJOR ? BK * ld : BK;
     }
-}
+
+    // The next slice, of which `left` inner indices exist.  Others, and rows past
+    // the last, read as (0, 0); they are never used for a stored output nor for a
+    // term beyond k.
+    __device__ __forceinline__ void load(int left, float2 (&v)[L])
+    {
+#pragma unroll
+        for (int s = 0; s < L; ++s) {
+            const bool in = KMAJOR ? row < rows && inner + s * kStep < left : row + s * kStep < rows && inner < left;
+            v[s] = in ? __ldg(p + s * stride) : make_float2(0.0f, 0.0f);
+        }
+        p += advance;
+    }
+};
 
 template <int N, int BK, int T, int L, int LD, bool KMAJOR>
 __device__ __forceinline__ void store_slice(float2 (*S)[LD], const float2 (&v)[L])
@@ -111,6 +130,9 @@ gemm_kernel(const float2* __restrict__ A, const float2* __restrict__ B, float2* 
     const int tx = threadIdx.x % S::TX;
     const int ty = threadIdx.x / S::TX;
     const int64_t nslices = (d.k + S::BK - 1) / S::BK;
+    // A slice is unrolled to about 1,400 instructions at most: the fully unrolled
+    // slice of the 4 x 4 sub-tile overflows the instruction cache.
+    constexpr int U = 32 / (S::TM * S::TN) < 8 ? 32 / (S::TM * S::TN) : 8;
 
     for (int64_t tile = blockIdx.x; tile < d.tiles; tile += gridDim.x) {
         const int64_t i0 = (tile / d.tiles_n) * S::BM;
@@ -122,9 +144,13 @@ gemm_kernel(const float2* __restrict__ A, const float2* __restrict__ B, float2* 
             for (int c = 0; c < S::TN; ++c) acc[r][c] = make_float2(0.0f, 0.0f);
 
         float2 va[S::LA], vb[S::LB];
+        Slices<S::BM, S::BK, S::T, S::LA, TA> slices_a(A, d.lda, d.m, i0);
+        Slices<S::BN, S::BK, S::T, S::LB, !TB> slices_b(B, d.ldb, d.n, j0);
         auto load = [&](int64_t sl) {
-            load_slice<S::BM, S::BK, S::T, S::LA, TA>(A, d.lda, d.m, d.k, i0, sl * S::BK, va);
-            load_slice<S::BN, S::BK, S::T, S::LB, !TB>(B, d.ldb, d.n, d.k, j0, sl * S::BK, vb);
+            const int64_t rest = d.k - sl * S::BK;
+            const int left = static_cast<int>(rest < S::BK ? rest : S::BK);
+            slices_a.load(left, va);
+            slices_b.load(left, vb);
         };
         // to shared memory; true when every value this thread loaded is normalised
         auto store = [&](int buf) {
@@ -154,15 +180,19 @@ gemm_kernel(const float2* __restrict__ A, const float2* __restrict__ B, float2* 
 #pragma unroll 1
                 for (int kk = 0; kk < kn; ++kk) step<S, false>(As[cur][kk], Bs[cur][kk], ty, tx, acc);
             } else if (kn == S::BK) {
-                // Unrolled to about 1,400 instructions at most: the fully
-                // unrolled slice of the 4 x 4 sub-tile overflows the
-                // instruction cache.
-                constexpr int U = 32 / (S::TM * S::TN) < 8 ? 32 / (S::TM * S::TN) : 8;
 #pragma unroll U
                 for (int kk = 0; kk < S::BK; ++kk) step<S, true>(As[cur][kk], Bs[cur][kk], ty, tx, acc);
             } else {
+                // a last slice of fewer inner indices; one loop for both lengths
+                // costs 1% on the whole slices
+                int kk = 0;
 #pragma unroll 1
-                for (int kk = 0; kk < kn; ++kk) step<S, true>(As[cur][kk], Bs[cur][kk], ty, tx, acc);
+                for (; kk + U <= kn; kk += U) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) step<S, true>(As[cur][kk + u], Bs[cur][kk + u], ty, tx, acc);
+                }
+#pragma unroll 1
+                for (; kk < kn; ++kk) step<S, true>(As[cur][kk], Bs[cur][kk], ty, tx, acc);
             }
             ok = more ? store(cur ^ 1) : true;
             fast = __syncthreads_and(ok);
@@ -204,15 +234,19 @@ ff_status launch(bool ta, bool tb, const float2* A, const float2* B, float2* C, 
 // outputs only, and the time is that of the SM with the most tiles: measured
 // cycles per inner index with q tiles on an SM are close to  a q + b  (a: the
 // tile's outputs per lane times the cycles per term, which grow as the tile's
-// operand reuse shrinks: 26.2, 27.7, 30.5 and 33.7; b: the part of a chain's
+// operand reuse shrinks: 25.1, 26.4, 27.6 and 30.2; b: the part of a chain's
 // latency that the few resident warps leave uncovered).  The shape with the
 // least of it runs.  500 x 300 x 700: 392 us with 64 x 64 tiles alone (40 of
-// 152 SMs busy), 90 us; 100 x 100 x 1000: 508 -> 35 us; 1024^3: 1042 -> 769
+// 152 SMs busy), 82 us; 100 x 100 x 1000: 508 -> 29 us; 1024^3: 1042 -> 737
 // us; from about 2048 rows and columns the largest tile is always taken.
+//
+// The small tiles do few terms per inner index, so the work of one slice (its
+// loads, stores and barrier) is spread over 64 of them: 90 us at 500 x 300 x 700
+// with slices of 16, 82 with 64.  64 x 64 tiles gain nothing from deeper slices.
 using Tile64 = Tile<64, 64, 4, 4, 16, 2>;
 using Tile32 = Tile<32, 32, 2, 2, 32, 2>;
-using Tile16 = Tile<16, 16, 1, 2, 16, 8>;
-using Tile8 = Tile<8, 16, 1, 1, 32, 8>;
+using Tile16 = Tile<16, 16, 1, 2, 64, 4>;
+using Tile8 = Tile<8, 16, 1, 1, 64, 4>;
 
 template <class S>
 double cycles(int64_t m, int64_t n, int sm_count, double a, double b)
@@ -224,10 +258,10 @@ double cycles(int64_t m, int64_t n, int sm_count, double a, double b)
 ff_status launch_best(bool ta, bool tb, const float2* A, const float2* B, float2* C, const Dims& d, int sm_count,
                       cudaStream_t s)
 {
-    const double c64 = cycles<Tile64>(d.m, d.n, sm_count, 838.0, 30.0);
-    const double c32 = cycles<Tile32>(d.m, d.n, sm_count, 222.0, 20.0);
-    const double c16 = cycles<Tile16>(d.m, d.n, sm_count, 61.0, 25.0);
-    const double c8 = cycles<Tile8>(d.m, d.n, sm_count, 33.7, 30.0);
+    const double c64 = cycles<Tile64>(d.m, d.n, sm_count, 803.0, 45.0);
+    const double c32 = cycles<Tile32>(d.m, d.n, sm_count, 211.0, 20.0);
+    const double c16 = cycles<Tile16>(d.m, d.n, sm_count, 55.2, 28.0);
+    const double c8 = cycles<Tile8>(d.m, d.n, sm_count, 30.2, 28.0);
     const double best = std::fmin(std::fmin(c64, c32), std::fmin(c16, c8));
     if (best == c64) return launch<Tile64>(ta, tb, A, B, C, d, s);
     if (best == c32) return launch<Tile32>(ta, tb, A, B, C, d, s);

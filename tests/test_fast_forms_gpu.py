@@ -73,6 +73,23 @@ def test_gemm_tiles(m, n, k, kind):
             same_bits(got.cpu().numpy(), want)
 
 
+# inner lengths around a whole slice of the two small tiles and of a group of
+# its steps, for each operand layout; one value off the fast forms in the first
+# slice only, so that later slices switch back
+@pytest.mark.parametrize("m,n", [(33, 65), (250, 255)])
+@pytest.mark.parametrize("k", [1, 7, 63, 64, 65, 72, 127, 129, 200])
+def test_gemm_slices(m, n, k):
+    g = inputs.gemm(m, n, k, inputs.seed_for(6, 61))
+    A, B = g.A.clone(), g.B
+    A[m // 2, 0, 1] = A[m // 2, 0, 0]
+    At, Bt = A.permute(1, 0, 2).contiguous(), B.permute(1, 0, 2).contiguous()
+    want = oracle.gemm(A.numpy(), B.numpy())
+    for ta in (False, True):
+        for tb in (False, True):
+            got = ff.gemm((At if ta else A).to(DEV), (Bt if tb else B).to(DEV), transa=ta, transb=tb)
+            same_bits(got.cpu().numpy(), want)
+
+
 # one warp per row and right-hand side (few rows), pairs, and tiles of 2, 3 + 2,
 # 3, 4 and 4 + 3; row lengths around the loads in flight, even and odd
 FORWARD = [(40, 1100, 1), (40, 515, 3), (700, 130, 4), (700, 67, 3), (650, 70, 9), (1300, 66, 2), (1300, 33, 3), (1230, 131, 5),

@@ -23,7 +23,19 @@
 //      ticket back to zero (the caller zeroes a workspace once, before its
 //      first use, so a call is a single launch).
 // No block ever waits for another.
+//
+// Large n is bound by HBM (ff_dot at 2^28: 7.27 TB/s).  Below a few million
+// values the time is a chain of latencies: one round of loads, the trees, and
+// the last block's turn (partial stored, ticket, partials read).  So a thread's
+// loads are issued together wherever the grid covers the vector with one group
+// per thread, single values outside the chunks are prefetched, the ticket's
+// atomic carries the ordering itself instead of two full fences, and the float-
+// float sums, which are normalised, close with Fast2Sum (ff_core.cuh).  ff_dot2,
+// 3,000,001 values from HBM: 9.3 -> 7.1 us; ff_sum2 8.0 -> 5.8; ff_dot at
+// 100,003 6.0 -> 5.1, at 10^6 7.6 -> 6.5; on mixed offsets at 2^26 192 -> 155
+// (values one by one before, four together now).
 #include <mutex>
+#include <type_traits>
 
 #include "ff_core.cuh"
 #include "ff_host.cuh"
@@ -32,21 +44,28 @@ namespace {
 
 constexpr int kRBlock = 256;
 constexpr int kRWarps = kRBlock / 32;
+constexpr int kPartials = 4;   // block values that a thread of the last block loads together
 // Resident 256-thread blocks per SM at most: a read-only stream reaches a
 // higher DRAM rate with moderate residency than with every SM full (ff_sum
 // at 2^26 / 2^28: 0.97 / 1.02 of the measured copy rate with 8 blocks,
-// 0.995 / 1.06 with 6; ff_dot is held at 6 by its registers either way).
+// 0.995 / 1.06 with 6).
 constexpr int kRMaxBlocksPerSm = 6;
 constexpr size_t kPartialsOffset = 256;  // ticket at offset 0, partials at 256
 
+// kBlocksPerSm, kOneBlocksPerSm: the register budgets of the two kernels below
+// (the one-group kernel holds a whole group: 48 registers, five blocks; the
+// loop built the same way took 60, four blocks, and 601 us for ff_dot at 2^28
+// against 591 with 40).
 struct FFSum {
     using T = float2;
     using Acc = float2;
+    static constexpr int kBlocksPerSm = 6, kOneBlocksPerSm = 5;
     static constexpr bool kDot = false;
-    __device__ static Acc finalize(Acc a) { return a; }
+    __device__ static Acc finalize(Acc a) { return ffk::ff_overflow_lo(a); }
     __device__ static Acc zero() { return make_float2(0.0f, 0.0f); }
     __device__ static Acc step(Acc acc, T x, T) { return ffk::add22(acc, x); }
-    __device__ static Acc combine(Acc a, Acc b) { return ffk::add22(a, b); }
+    // sums are Add22 results, so normalised: Fast2Sum closes with the same bits
+    __device__ static Acc combine(Acc a, Acc b) { return ffk::add22_fast(a, b); }
     __device__ static Acc shfl_down(Acc v, int off)
     {
         return make_float2(__shfl_down_sync(0xffffffffu, v.x, off), __shfl_down_sync(0xffffffffu, v.y, off));
@@ -55,12 +74,13 @@ struct FFSum {
 
 struct FFDot : FFSum {
     static constexpr bool kDot = true;
-    __device__ static Acc step(Acc acc, T x, T y) { return ffk::add22(acc, ffk::mul22(x, y)); }
+    __device__ static Acc step(Acc acc, T x, T y) { return ffk::add22_fast(acc, ffk::mul22(x, y)); }
 };
 
 struct F64Dot {
     using T = double;
     using Acc = double;
+    static constexpr int kBlocksPerSm = 5, kOneBlocksPerSm = 4;
     static constexpr bool kDot = true;
     __device__ static Acc finalize(Acc a) { return a; }
     __device__ static Acc zero() { return 0.0; }
@@ -78,6 +98,7 @@ struct F64Dot {
 struct F32Sum2 {
     using T = float;
     using Acc = float2;  // (p, s)
+    static constexpr int kBlocksPerSm = 6, kOneBlocksPerSm = 5;
     static constexpr bool kDot = false;
     __device__ static Acc zero() { return make_float2(0.0f, 0.0f); }
     __device__ static Acc step(Acc a, T x, T)
@@ -147,121 +168,156 @@ __device__ __forceinline__ typename P::Acc block_reduce(typename P::Acc v, typen
 #pragma unroll
         for (int off = kRWarps / 2; off > 0; off >>= 1) v = P::combine(v, P::shfl_down(v, off));
     }
-    __syncthreads();
     return v;
 }
 
-template <class P, int U>
-__global__ void __launch_bounds__(kRBlock)
+// Counts this block in and returns how many came before it.  The addition
+// releases the block's partial (thread 0 stored it) and acquires those counted
+// before.
+__device__ __forceinline__ unsigned arrive(unsigned* ticket)
+{
+    unsigned before;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(ticket) : "memory");
+    return before;
+}
+
+// Steps 2-4 for this block's thread values.
+template <class P>
+__device__ __forceinline__ void combine_blocks(typename P::Acc acc, typename P::Acc* out, typename P::Acc* partials,
+                                               unsigned* ticket)
+{
+    using Acc = typename P::Acc;
+    __shared__ Acc sm[kRWarps];
+    __shared__ bool is_last;
+    acc = block_reduce<P>(acc, sm);
+    if (gridDim.x == 1) {
+        if (threadIdx.x == 0) *out = P::finalize(acc);
+        return;
+    }
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = acc;
+        is_last = arrive(ticket) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!is_last) return;
+    Acc a2 = P::zero();
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += kPartials * kRBlock) {
+        Acc v[kPartials];
+#pragma unroll
+        for (int u = 0; u < kPartials; ++u)
+            if (b + u * kRBlock < gridDim.x) v[u] = __ldcg(partials + b + u * kRBlock);
+#pragma unroll
+        for (int u = 0; u < kPartials; ++u)
+            if (b + u * kRBlock < gridDim.x) a2 = P::combine(a2, v[u]);
+    }
+    a2 = block_reduce<P>(a2, sm);
+    if (threadIdx.x == 0) {
+        *out = P::finalize(a2);
+        *ticket = 0u;
+    }
+}
+
+// Brings a value that thread 0 needs after its chunks to the caches early.
+__device__ __forceinline__ void prefetch(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
+// A thread's first values (thread 0), chunks and last values (thread 0).
+// ONE: the grid has a thread for every U chunks, so a thread makes one group of
+// at most U, loaded together.  Otherwise groups of U and single chunks follow
+// one another.
+template <class P, int U, bool ONE>
+__global__ void __launch_bounds__(kRBlock, ONE ? P::kOneBlocksPerSm : P::kBlocksPerSm)
 reduce_kernel(const typename P::T* x, const typename P::T* y, size_t n, int head, typename P::Acc* out,
               typename P::Acc* partials, unsigned* ticket)
 {
     using T = typename P::T;
     using Acc = typename P::Acc;
     using V = typename V16<T>::V;
-    __shared__ Acc sm[kRWarps];
-    __shared__ bool is_last;
-
+    using Index = std::conditional_t<ONE, unsigned, size_t>;
     constexpr int E = V16<T>::E;
-    const size_t tid = static_cast<size_t>(blockIdx.x) * kRBlock + threadIdx.x;
-    const size_t nthr = static_cast<size_t>(gridDim.x) * kRBlock;
+    const Index tid = static_cast<Index>(blockIdx.x) * kRBlock + threadIdx.x;
+    const Index nthr = static_cast<Index>(gridDim.x) * kRBlock;
     const size_t h = static_cast<size_t>(head);
-    const size_t nv = (n - h) / E;
+    const Index nv = static_cast<Index>((n - h) / E);
+    const size_t tail = h + static_cast<size_t>(nv) * E;
 
     Acc acc = P::zero();
-    if (tid == 0)
-        for (size_t j = 0; j < h; ++j) acc = P::step(acc, x[j], P::kDot ? y[j] : T());
-
-    const V* xv = reinterpret_cast<const V*>(x + h);
-    const V* yv = reinterpret_cast<const V*>((P::kDot ? y : x) + h);
-    size_t i = tid;
-    for (; i + (U - 1) * nthr < nv; i += U * nthr) {
-        V xs[U], ys[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            xs[u] = __ldcs(xv + i + u * nthr);
-            if (P::kDot) ys[u] = __ldcs(yv + i + u * nthr);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            T xe[E], ye[E];
-            split_vec(xs[u], xe);
-            if (P::kDot) split_vec(ys[u], ye);
-#pragma unroll
-            for (int e = 0; e < E; ++e) acc = P::step(acc, xe[e], P::kDot ? ye[e] : T());
-        }
-    }
-    for (; i < nv; i += nthr) {
-        V xs, ys;
-        xs = __ldcs(xv + i);
-        if (P::kDot) ys = __ldcs(yv + i);
+    auto values = [&](size_t j0, size_t j1) {
+        for (size_t j = j0; j < j1; ++j) acc = P::step(acc, x[j], P::kDot ? y[j] : T());
+    };
+    auto chunk = [&](const V& xs, const V& ys) {
         T xe[E], ye[E];
         split_vec(xs, xe);
         if (P::kDot) split_vec(ys, ye);
 #pragma unroll
         for (int e = 0; e < E; ++e) acc = P::step(acc, xe[e], P::kDot ? ye[e] : T());
+    };
+    if (tid == 0 && tail < n) {
+        prefetch(x + tail);
+        if (P::kDot) prefetch(y + tail);
     }
-    if (tid == 0)
-        for (size_t j = h + nv * E; j < n; ++j) acc = P::step(acc, x[j], P::kDot ? y[j] : T());
-
-    acc = block_reduce<P>(acc, sm);
-    if (gridDim.x == 1) {
-        if (threadIdx.x == 0) *out = P::finalize(acc);
-        return;
+    const V* xv = reinterpret_cast<const V*>(x + h);
+    const V* yv = reinterpret_cast<const V*>((P::kDot ? y : x) + h);
+    Index i = tid;
+    if constexpr (ONE) {
+        V xs[U], ys[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u * nthr < nv) {
+                xs[u] = __ldcs(xv + (i + u * nthr));
+                if (P::kDot) ys[u] = __ldcs(yv + (i + u * nthr));
+            }
+        if (tid == 0) values(0, h);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u * nthr < nv) chunk(xs[u], ys[u]);
+    } else {
+        if (tid == 0) values(0, h);
+        for (; i + (U - 1) * nthr < nv; i += U * nthr) {
+            V xs[U], ys[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                xs[u] = __ldcs(xv + i + u * nthr);
+                if (P::kDot) ys[u] = __ldcs(yv + i + u * nthr);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) chunk(xs[u], ys[u]);
+        }
+        for (; i < nv; i += nthr) {
+            const V xs = __ldcs(xv + i);
+            V ys = xs;
+            if (P::kDot) ys = __ldcs(yv + i);
+            chunk(xs, ys);
+        }
     }
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = acc;
-        __threadfence();
-        const unsigned t = atomicAdd(ticket, 1u);
-        is_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    Acc a2 = P::zero();
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += kRBlock) a2 = P::combine(a2, __ldcg(partials + b));
-    a2 = block_reduce<P>(a2, sm);
-    if (threadIdx.x == 0) {
-        *out = P::finalize(a2);
-        *ticket = 0u;
-    }
+    if (tid == 0) values(tail, n);
+    combine_blocks<P>(acc, out, partials, ticket);
 }
 
 // Unaligned operands (offsets modulo 16 differ): scalar loads, same tree.
-template <class P>
+template <class P, int U>
 __global__ void __launch_bounds__(kRBlock)
 reduce_scalar_kernel(const typename P::T* x, const typename P::T* y, size_t n, typename P::Acc* out,
                      typename P::Acc* partials, unsigned* ticket)
 {
     using T = typename P::T;
     using Acc = typename P::Acc;
-    __shared__ Acc sm[kRWarps];
-    __shared__ bool is_last;
     const size_t tid = static_cast<size_t>(blockIdx.x) * kRBlock + threadIdx.x;
     const size_t nthr = static_cast<size_t>(gridDim.x) * kRBlock;
     Acc acc = P::zero();
-    for (size_t i = tid; i < n; i += nthr) acc = P::step(acc, x[i], P::kDot ? y[i] : T());
-    acc = block_reduce<P>(acc, sm);
-    if (gridDim.x == 1) {
-        if (threadIdx.x == 0) *out = P::finalize(acc);
-        return;
+    for (size_t i = tid; i < n; i += U * nthr) {   // U values loaded together
+        T xs[U], ys[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (i + u * nthr < n) {
+                xs[u] = __ldcs(x + i + u * nthr);
+                if (P::kDot) ys[u] = __ldcs(y + i + u * nthr);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u * nthr < n) acc = P::step(acc, xs[u], P::kDot ? ys[u] : T());
     }
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = acc;
-        __threadfence();
-        const unsigned t = atomicAdd(ticket, 1u);
-        is_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    Acc a2 = P::zero();
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += kRBlock) a2 = P::combine(a2, __ldcg(partials + b));
-    a2 = block_reduce<P>(a2, sm);
-    if (threadIdx.x == 0) {
-        *out = P::finalize(a2);
-        *ticket = 0u;
-    }
+    combine_blocks<P>(acc, out, partials, ticket);
 }
 
 constexpr int kU = 4;
@@ -273,7 +329,7 @@ size_t workspace_bytes(const ffh::DeviceInfo& di) { return kPartialsOffset + max
 struct Shape {
     unsigned grid;
     int head;
-    bool vec;
+    bool vec, one;
 };
 
 template <class P>
@@ -289,20 +345,35 @@ Shape shape_for(const typename P::T* x, const typename P::T* y, size_t n, const 
         constexpr int E = V16<T>::E;
         sh.head = px != 0 ? static_cast<int>((16u - px) / sizeof(T)) : 0;
         if (static_cast<size_t>(sh.head) > n) sh.head = static_cast<int>(n);
-        const void* kern = reinterpret_cast<const void*>(&reduce_kernel<P, kU>);
+        const void* kern = reinterpret_cast<const void*>(&reduce_kernel<P, kU, false>);
         int occ = ffh::occupancy(kern, kRBlock);
         if (occ > kRMaxBlocksPerSm) occ = kRMaxBlocksPerSm;
         const size_t nv = n > static_cast<size_t>(sh.head) ? (n - sh.head) / E : 0;
         sh.grid = ffh::grid_for(nv, static_cast<size_t>(kRBlock) * kU, di.sm_count, occ);
+        sh.one = sh.grid <= static_cast<unsigned>(di.sm_count) * P::kOneBlocksPerSm &&
+                 static_cast<size_t>(sh.grid) * kRBlock * kU >= nv;
     } else {
         sh.head = 0;
-        const void* kern = reinterpret_cast<const void*>(&reduce_scalar_kernel<P>);
+        const void* kern = reinterpret_cast<const void*>(&reduce_scalar_kernel<P, kU>);
         int occ = ffh::occupancy(kern, kRBlock);
         if (occ > kRMaxBlocksPerSm) occ = kRMaxBlocksPerSm;
         sh.grid = ffh::grid_for(n, static_cast<size_t>(kRBlock) * kU, di.sm_count, occ);
     }
     if (sh.grid > cap) sh.grid = static_cast<unsigned>(cap);
     return sh;
+}
+
+template <class P>
+ff_status launch(const Shape& sh, const typename P::T* x, const typename P::T* y, size_t n, typename P::Acc* out,
+                 typename P::Acc* partials, unsigned* ticket, cudaStream_t s)
+{
+    if (sh.one)
+        reduce_kernel<P, kU, true><<<sh.grid, kRBlock, 0, s>>>(x, y, n, sh.head, out, partials, ticket);
+    else if (sh.vec)
+        reduce_kernel<P, kU, false><<<sh.grid, kRBlock, 0, s>>>(x, y, n, sh.head, out, partials, ticket);
+    else
+        reduce_scalar_kernel<P, kU><<<sh.grid, kRBlock, 0, s>>>(x, y, n, out, partials, ticket);
+    return ffh::check_launch();
 }
 
 template <class P>
@@ -323,11 +394,7 @@ ff_status run_reduce(const typename P::T* x, const typename P::T* y, size_t n, t
     const Shape sh = shape_for<P>(x, y, n, di);
     // No clearing launch: the ticket is zero on entry (the workspace contract)
     // and the last block resets it to zero before the kernel ends.
-    if (sh.vec)
-        reduce_kernel<P, kU><<<sh.grid, kRBlock, 0, s>>>(x, y, n, sh.head, out, partials, ticket);
-    else
-        reduce_scalar_kernel<P><<<sh.grid, kRBlock, 0, s>>>(x, y, n, out, partials, ticket);
-    return ffh::check_launch();
+    return launch<P>(sh, x, y, n, out, partials, ticket, s);
 }
 
 }  // namespace
@@ -460,9 +527,5 @@ extern "C" ff_status ff_dot_noalloc(const ff2* x_, const ff2* y_, size_t n, ff2*
         st = ffh::cuda_status(cudaMemsetAsync(ticket, 0, sizeof(unsigned), s));
         if (st != FF_OK) return st;
     }
-    if (sh.vec)
-        reduce_kernel<FFDot, kU><<<sh.grid, kRBlock, 0, s>>>(x, y, n, sh.head, out, partials, ticket);
-    else
-        reduce_scalar_kernel<FFDot><<<sh.grid, kRBlock, 0, s>>>(x, y, n, out, partials, ticket);
-    return ffh::check_launch();
+    return launch<FFDot>(sh, x, y, n, out, partials, ticket, s);
 }

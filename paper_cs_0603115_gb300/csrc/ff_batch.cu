@@ -357,7 +357,7 @@ batch_kernel(const DevInst* __restrict__ insts, const Tile* __restrict__ tiles, 
     int pending = -1, parity = 0; // instance of the last multi-tile dot whose arrival was not looked at yet
     bool ended = false;           // thread 0: it ended that instance
 
-    int64_t t = blockIdx.x;
+    int64_t t = blockIdx.x + ffk::prior_kernel_done();
     Tile tl = t < ntiles ? tiles[t] : Tile{0, 0, 0};
     for (; t < ntiles; t += gridDim.x) {
         const Tile cur = tl;
@@ -464,8 +464,9 @@ batch_gemv_kernel(const DevInst* __restrict__ insts, const Tile* __restrict__ ti
         const DevInst& I = insts[tl.inst];
         gemv_rows_tile_body<kRowPairs>(I.x, I.y, I.out, I.n, I.lda, I.m, I.vec, I.rows_per_warp, tl.start);
     };
+    const unsigned first = blockIdx.x + ffk::prior_kernel_done();
     if (next == nullptr) {   // a block per tile
-        tile(blockIdx.x);
+        tile(first);
         return;
     }
     __shared__ unsigned long long s_t;
@@ -751,9 +752,8 @@ ff_status ff_batch_run(const ff_batch_plan* p, void* ws, size_t ws_bytes, cudaSt
     } else {
         next = nullptr;
     }
-    kernel_for(*var, *p)<<<p->grid, p->tune.block, 0, s>>>(p->d_inst, p->d_tiles, p->ntiles, partials, counters,
-                                                           next);
-    return ffh::check_launch();
+    return ffh::launch_kernel(kernel_for(*var, *p), p->grid, static_cast<unsigned>(p->tune.block), s, p->d_inst, p->d_tiles,
+                              p->ntiles, partials, counters, next);
 }
 
 void ff_batch_plan_destroy(ff_batch_plan* p)

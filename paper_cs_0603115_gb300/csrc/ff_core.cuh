@@ -11,6 +11,17 @@
 
 namespace ffk {
 
+// Waits until the kernels before this one in the stream have ended and their
+// writes are visible (nothing to wait for unless the launch allowed overlap), and
+// returns 0.  First in every kernel; the addresses of all reads are formed with
+// the result, so that no read of read-only data is moved above the wait.
+__device__ __forceinline__ unsigned prior_kernel_done()
+{
+    unsigned zero;
+    asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero)::"memory");
+    return zero;
+}
+
 // Add12 theorem (Knuth): s = a (+) b, r = (a + b) - s exactly; branch free.
 __device__ __forceinline__ float2 add12(float a, float b)
 {

@@ -134,7 +134,7 @@ gemm_kernel(const float2* __restrict__ A, const float2* __restrict__ B, float2* 
     // slice of the 4 x 4 sub-tile overflows the instruction cache.
     constexpr int U = 32 / (S::TM * S::TN) < 8 ? 32 / (S::TM * S::TN) : 8;
 
-    for (int64_t tile = blockIdx.x; tile < d.tiles; tile += gridDim.x) {
+    for (int64_t tile = blockIdx.x + ffk::prior_kernel_done(); tile < d.tiles; tile += gridDim.x) {
         const int64_t i0 = (tile / d.tiles_n) * S::BM;
         const int64_t j0 = (tile % d.tiles_n) * S::BN;
         float2 acc[S::TM][S::TN];
@@ -219,15 +219,9 @@ ff_status launch(bool ta, bool tb, const float2* A, const float2* B, float2* C, 
     // one block per tile up to the 1-D grid limit; blocks loop over the rest
     const int64_t cap = 0x7fffffffLL;
     const unsigned grid = static_cast<unsigned>(d.tiles < cap ? d.tiles : cap);
-    if (!ta && !tb)
-        gemm_kernel<S, false, false><<<grid, S::T, 0, s>>>(A, B, C, d);
-    else if (ta && !tb)
-        gemm_kernel<S, true, false><<<grid, S::T, 0, s>>>(A, B, C, d);
-    else if (!ta && tb)
-        gemm_kernel<S, false, true><<<grid, S::T, 0, s>>>(A, B, C, d);
-    else
-        gemm_kernel<S, true, true><<<grid, S::T, 0, s>>>(A, B, C, d);
-    return ffh::check_launch();
+    const auto kernel = ta ? (tb ? &gemm_kernel<S, true, true> : &gemm_kernel<S, true, false>)
+                           : (tb ? &gemm_kernel<S, false, true> : &gemm_kernel<S, false, false>);
+    return ffh::launch_kernel(kernel, grid, S::T, s, A, B, C, d);
 }
 
 // Tile choice.  Every output is one serial chain of k terms, so C is cut by

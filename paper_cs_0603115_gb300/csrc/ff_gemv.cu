@@ -204,9 +204,11 @@ __global__ void __launch_bounds__(32 * kFWarps, MINB)
 gemv_kernel(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda, const float2* __restrict__ X,
             int64_t ldx, float2* __restrict__ Y, int64_t ldy, int na)
 {
-    const int64_t r = static_cast<int64_t>(blockIdx.x) * kFWarps + (threadIdx.x >> 5);
+    const unsigned zero = ffk::prior_kernel_done();
+    const int64_t r = static_cast<int64_t>(blockIdx.x + zero) * kFWarps + (threadIdx.x >> 5);
     if (r >= m) return;
     const int y = blockIdx.y;
+    X += zero;
     if (KA == KB || y < na) {
         const int64_t c0 = static_cast<int64_t>(y) * KA;
         gemv_row<KA, VEC, U, PIPE>(A + r * lda, X + c0 * ldx, n, ldx, Y + c0 * ldy + r, ldy);
@@ -243,9 +245,8 @@ ff_status launch_gemv(const TileSplit& t, const float2* A, int64_t m, int64_t n,
                       int64_t ldx, float2* Y, int64_t ldy, cudaStream_t s)
 {
     const dim3 grid(static_cast<unsigned>((m + kFWarps - 1) / kFWarps), static_cast<unsigned>(t.na + t.nb));
-    gemv_kernel<KA, KB, VEC, U, PIPE, MINB><<<grid, 32 * kFWarps, 0, s>>>(A, m, n, lda, X, ldx, Y, ldy,
-                                                                         static_cast<int>(t.na));
-    return ffh::check_launch();
+    return ffh::launch_kernel(&gemv_kernel<KA, KB, VEC, U, PIPE, MINB>, grid, 32 * kFWarps, s, A, m, n, lda, X, ldx, Y,
+                              ldy, static_cast<int>(t.na));
 }
 
 // Chunks in flight (U) and the register budget that lets the compiler issue
@@ -339,13 +340,13 @@ template <int KT, int E, int R>
 __device__ __forceinline__ void gemv_t_tile(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda,
                                             const float2* __restrict__ dY, int64_t lddy, int64_t rpb, int64_t nrb,
                                             int cx, float2* __restrict__ out, int64_t out_ld, int64_t rb_stride,
-                                            float2 (*part)[kGBlock])
+                                            float2 (*part)[kGBlock], unsigned zero)
 {
     const int tx = threadIdx.x & (cx - 1);
     const int ty = threadIdx.x / cx;
     const int rg = kGBlock / cx;
-    const int64_t j = (static_cast<int64_t>(blockIdx.x) * cx + tx) * E;   // first column
-    const int64_t rb = static_cast<int64_t>(blockIdx.y) * rg + ty;
+    const int64_t j = (static_cast<int64_t>(blockIdx.x + zero) * cx + tx) * E;   // first column
+    const int64_t rb = static_cast<int64_t>(blockIdx.y + zero) * rg + ty;
     const int64_t r0 = rb * rpb;
     const int64_t r1 = r0 + rpb < m ? r0 + rpb : m;
     float2 acc[KT][E];
@@ -392,15 +393,16 @@ gemv_t_kernel(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda, c
               int64_t rb_stride, int na)
 {
     __shared__ float2 part[KA * E][kGBlock];
+    const unsigned zero = ffk::prior_kernel_done();
     const int z = blockIdx.z;
     if (KA == KB || z < na) {
         const int64_t c0 = static_cast<int64_t>(z) * KA;
         gemv_t_tile<KA, E, R>(A, m, n, lda, dY + c0 * lddy, lddy, rpb, nrb, cx, out + c0 * out_ld, out_ld, rb_stride,
-                              part);
+                              part, zero);
     } else {
         const int64_t c0 = static_cast<int64_t>(na) * KA + static_cast<int64_t>(z - na) * KB;
         gemv_t_tile<KB, E, R>(A, m, n, lda, dY + c0 * lddy, lddy, rpb, nrb, cx, out + c0 * out_ld, out_ld, rb_stride,
-                              part);
+                              part, zero);
     }
 }
 
@@ -409,7 +411,7 @@ __global__ void __launch_bounds__(kGBlock)
 gemv_t_combine(const float2* __restrict__ ws, int64_t n, int64_t k, int64_t nrb, float2* __restrict__ dX,
                int64_t lddx)
 {
-    const int64_t idx = static_cast<int64_t>(blockIdx.x) * kGBlock + threadIdx.x;
+    const int64_t idx = static_cast<int64_t>(blockIdx.x + ffk::prior_kernel_done()) * kGBlock + threadIdx.x;
     if (idx >= n * k) return;
     const int64_t c = idx / n, j = idx - c * n;
     float2 acc = ws[c * n + j];
@@ -548,9 +550,8 @@ ff_status launch_adjoint(const AdjointPlan& p, const TileSplit& t, const float2*
     const int64_t cols = n / E;
     const dim3 grid(static_cast<unsigned>((cols + p.cx - 1) / p.cx), static_cast<unsigned>(p.gy),
                     static_cast<unsigned>(t.na + t.nb));
-    gemv_t_kernel<KA, KB, E, R, MINB><<<grid, kGBlock, 0, s>>>(A, m, n, lda, dY, lddy, p.rpb, p.nrb, p.cx, out, out_ld,
-                                                               rb_stride, static_cast<int>(t.na));
-    return ffh::check_launch();
+    return ffh::launch_kernel(&gemv_t_kernel<KA, KB, E, R, MINB>, grid, kGBlock, s, A, m, n, lda, dY, lddy, p.rpb, p.nrb,
+                              p.cx, out, out_ld, rb_stride, static_cast<int>(t.na));
 }
 
 // ---------------------------------------------------------------------------
@@ -583,9 +584,10 @@ gemv_dA_small_kernel(const float2* __restrict__ dY, int64_t m, int64_t lddy, con
     using V = std::conditional_t<E == 2, float4, float2>;
     constexpr int RS = 4 / E;   // rows per step
     __shared__ __align__(16) float2 sdy[KT][kTChunk];
-    const int64_t j_raw = (static_cast<int64_t>(blockIdx.x) * kGBlock + threadIdx.x) * E;
+    const unsigned zero = ffk::prior_kernel_done();
+    const int64_t j_raw = (static_cast<int64_t>(blockIdx.x + zero) * kGBlock + threadIdx.x) * E;
     const bool store = j_raw < n;
-    const int64_t j = store ? j_raw : n - E;
+    const int64_t j = store ? j_raw : n - E + zero;
     float2 x[KT][E];
     bool okx = true;
 #pragma unroll
@@ -596,7 +598,7 @@ gemv_dA_small_kernel(const float2* __restrict__ dY, int64_t m, int64_t lddy, con
 #pragma unroll
         for (int e = 0; e < E; ++e) okx &= ffk::normalised(x[c][e]);
     }
-    const int64_t r0 = static_cast<int64_t>(blockIdx.y) * rpb;
+    const int64_t r0 = static_cast<int64_t>(blockIdx.y + zero) * rpb;
     const int64_t r1 = r0 + rpb < m ? r0 + rpb : m;
 
     // R rows of the chunk from row q on
@@ -702,8 +704,7 @@ ff_status launch_dA(const float2* dY, int64_t m, int64_t lddy, const float2* X, 
     if (gy < 1) gy = 1;
     const int64_t rpb = ((m + gy - 1) / gy + RS - 1) / RS * RS;
     const dim3 grid(static_cast<unsigned>(col_blocks), static_cast<unsigned>((m + rpb - 1) / rpb));
-    gemv_dA_small_kernel<KT, E><<<grid, kGBlock, 0, s>>>(dY, m, lddy, X, n, ldx, dA, ldda, rpb);
-    return ffh::check_launch();
+    return ffh::launch_kernel(&gemv_dA_small_kernel<KT, E>, grid, kGBlock, s, dY, m, lddy, X, n, ldx, dA, ldda, rpb);
 }
 
 // k <= KT right-hand sides.
@@ -724,8 +725,10 @@ __global__ void __launch_bounds__(kGBlock)
 gemv_f64_kernel(const double* __restrict__ A, int64_t m, int64_t n, int64_t lda, const double* __restrict__ X,
                 int64_t ldx, double* __restrict__ Y, int64_t ldy)
 {
+    const unsigned zero = ffk::prior_kernel_done();
     const int lane = threadIdx.x & 31;
-    const int64_t r = static_cast<int64_t>(blockIdx.x) * kGWarps + (threadIdx.x >> 5);
+    const int64_t r = static_cast<int64_t>(blockIdx.x + zero) * kGWarps + (threadIdx.x >> 5);
+    X += zero;
     if (r >= m) return;
     double acc[KT];
 #pragma unroll
@@ -745,6 +748,13 @@ gemv_f64_kernel(const double* __restrict__ A, int64_t m, int64_t n, int64_t lda,
 #pragma unroll
         for (int c = 0; c < KT; ++c) Y[c * ldy + r] = acc[c];
     }
+}
+
+template <int KT>
+ff_status launch_f64(unsigned grid, const double* A, int64_t m, int64_t n, int64_t lda, const double* X, int64_t ldx,
+                     double* Y, int64_t ldy, cudaStream_t s)
+{
+    return ffh::launch_kernel(&gemv_f64_kernel<KT>, grid, kGBlock, s, A, m, n, lda, X, ldx, Y, ldy);
 }
 
 bool bad_dims(int64_t m, int64_t n, int64_t k) { return m < 0 || n < 0 || k < 1 || k > kMaxK; }
@@ -847,9 +857,8 @@ ff_status ff_gemv_t(const ff2* A_, int64_t m, int64_t n, int64_t lda, const ff2*
     if (st != FF_OK) return st;
     if (p.gy > 1) {
         const int64_t total = n * k;
-        gemv_t_combine<<<static_cast<unsigned>((total + kGBlock - 1) / kGBlock), kGBlock, 0, s>>>(
-            static_cast<float2*>(ws), n, k, p.nrb, dX, lddx);
-        st = ffh::check_launch();
+        st = ffh::launch_kernel(&gemv_t_combine, static_cast<unsigned>((total + kGBlock - 1) / kGBlock), kGBlock, s,
+                                static_cast<float2*>(ws), n, k, p.nrb, dX, lddx);
     }
     return st;
 }
@@ -891,14 +900,14 @@ ff_status ff_f64_gemv(const double* A, int64_t m, int64_t n, int64_t lda, const 
         const int kt = f64_tile_for(k - c0);
         const double* Xc = X + c0 * ldx;
         double* Yc = Y + c0 * ldy;
+        ff_status st = FF_OK;
         switch (kt) {
-        case 16: gemv_f64_kernel<16><<<grid, kGBlock, 0, s>>>(A, m, n, lda, Xc, ldx, Yc, ldy); break;
-        case 8: gemv_f64_kernel<8><<<grid, kGBlock, 0, s>>>(A, m, n, lda, Xc, ldx, Yc, ldy); break;
-        case 4: gemv_f64_kernel<4><<<grid, kGBlock, 0, s>>>(A, m, n, lda, Xc, ldx, Yc, ldy); break;
-        case 2: gemv_f64_kernel<2><<<grid, kGBlock, 0, s>>>(A, m, n, lda, Xc, ldx, Yc, ldy); break;
-        default: gemv_f64_kernel<1><<<grid, kGBlock, 0, s>>>(A, m, n, lda, Xc, ldx, Yc, ldy); break;
+        case 16: st = launch_f64<16>(grid, A, m, n, lda, Xc, ldx, Yc, ldy, s); break;
+        case 8: st = launch_f64<8>(grid, A, m, n, lda, Xc, ldx, Yc, ldy, s); break;
+        case 4: st = launch_f64<4>(grid, A, m, n, lda, Xc, ldx, Yc, ldy, s); break;
+        case 2: st = launch_f64<2>(grid, A, m, n, lda, Xc, ldx, Yc, ldy, s); break;
+        default: st = launch_f64<1>(grid, A, m, n, lda, Xc, ldx, Yc, ldy, s); break;
         }
-        ff_status st = ffh::check_launch();
         if (st != FF_OK) return st;
         c0 += kt;
     }

@@ -32,6 +32,32 @@ inline ff_status cuda_status(cudaError_t e)
     return FF_OK;
 }
 
+// Launches `kernel` so that it may be scheduled while the kernel before it in
+// the stream ends; every kernel launched here waits for that one's end itself,
+// before its first access to memory (ffk::prior_kernel_done).  Measured on
+// this GPU, a kernel launched the plain way behind another one completes on a
+// raster of 2.05 us and starts about 1.3 us late: 304 blocks that do nothing
+// take 4.10 us each, 1.43 launched this way; of 8.2 us, 5.2; of 53 us, 2 to 3 less.
+// A stream under capture records plain launches, so graphs hold plain edges.
+template <class... P, class... A>
+ff_status launch_kernel(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, A... args)
+{
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &capture);
+    if (e != cudaSuccess) (void)cudaGetLastError();   // the launch reports it
+    cudaLaunchAttribute overlap;
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = dim3(block);
+    c.stream = s;
+    c.attrs = &overlap;
+    c.numAttrs = e == cudaSuccess && capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    (void)cudaLaunchKernelEx(&c, kernel, P(args)...);
+    return check_launch();
+}
+
 inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 // A device array argument: non-NULL when it holds elements, 8-byte aligned.

@@ -234,7 +234,7 @@ reduce_kernel(const typename P::T* x, const typename P::T* y, size_t n, int head
     using V = typename V16<T>::V;
     using Index = std::conditional_t<ONE, unsigned, size_t>;
     constexpr int E = V16<T>::E;
-    const Index tid = static_cast<Index>(blockIdx.x) * kRBlock + threadIdx.x;
+    const Index tid = static_cast<Index>(blockIdx.x + ffk::prior_kernel_done()) * kRBlock + threadIdx.x;
     const Index nthr = static_cast<Index>(gridDim.x) * kRBlock;
     const size_t h = static_cast<size_t>(head);
     const Index nv = static_cast<Index>((n - h) / E);
@@ -266,12 +266,12 @@ reduce_kernel(const typename P::T* x, const typename P::T* y, size_t n, int head
                 xs[u] = __ldcs(xv + (i + u * nthr));
                 if (P::kDot) ys[u] = __ldcs(yv + (i + u * nthr));
             }
-        if (tid == 0) values(0, h);
+        if (tid == 0) values(tid, h);
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (i + u * nthr < nv) chunk(xs[u], ys[u]);
     } else {
-        if (tid == 0) values(0, h);
+        if (tid == 0) values(tid, h);
         for (; i + (U - 1) * nthr < nv; i += U * nthr) {
             V xs[U], ys[U];
 #pragma unroll
@@ -289,7 +289,7 @@ reduce_kernel(const typename P::T* x, const typename P::T* y, size_t n, int head
             chunk(xs, ys);
         }
     }
-    if (tid == 0) values(tail, n);
+    if (tid == 0) values(tail + tid, n);
     combine_blocks<P>(acc, out, partials, ticket);
 }
 
@@ -301,7 +301,7 @@ reduce_scalar_kernel(const typename P::T* x, const typename P::T* y, size_t n, t
 {
     using T = typename P::T;
     using Acc = typename P::Acc;
-    const size_t tid = static_cast<size_t>(blockIdx.x) * kRBlock + threadIdx.x;
+    const size_t tid = static_cast<size_t>(blockIdx.x + ffk::prior_kernel_done()) * kRBlock + threadIdx.x;
     const size_t nthr = static_cast<size_t>(gridDim.x) * kRBlock;
     Acc acc = P::zero();
     for (size_t i = tid; i < n; i += U * nthr) {   // U values loaded together
@@ -368,12 +368,10 @@ ff_status launch(const Shape& sh, const typename P::T* x, const typename P::T* y
                  typename P::Acc* partials, unsigned* ticket, cudaStream_t s)
 {
     if (sh.one)
-        reduce_kernel<P, kU, true><<<sh.grid, kRBlock, 0, s>>>(x, y, n, sh.head, out, partials, ticket);
-    else if (sh.vec)
-        reduce_kernel<P, kU, false><<<sh.grid, kRBlock, 0, s>>>(x, y, n, sh.head, out, partials, ticket);
-    else
-        reduce_scalar_kernel<P, kU><<<sh.grid, kRBlock, 0, s>>>(x, y, n, out, partials, ticket);
-    return ffh::check_launch();
+        return ffh::launch_kernel(&reduce_kernel<P, kU, true>, sh.grid, kRBlock, s, x, y, n, sh.head, out, partials, ticket);
+    if (sh.vec)
+        return ffh::launch_kernel(&reduce_kernel<P, kU, false>, sh.grid, kRBlock, s, x, y, n, sh.head, out, partials, ticket);
+    return ffh::launch_kernel(&reduce_scalar_kernel<P, kU>, sh.grid, kRBlock, s, x, y, n, out, partials, ticket);
 }
 
 template <class P>

@@ -24,6 +24,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "ff_core.cuh"
 #include "ff_host.cuh"
 
 namespace ffst {
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(kBlock) stream_vec(Args<T, NIN, NOUT> a, Op op
 {
     using V = typename Vec<T>::V;
     constexpr int E = Vec<T>::E;
-    const size_t tid = static_cast<size_t>(blockIdx.x) * kBlock + threadIdx.x;
+    const size_t tid = static_cast<size_t>(blockIdx.x + ffk::prior_kernel_done()) * kBlock + threadIdx.x;
     const size_t nthr = static_cast<size_t>(gridDim.x) * kBlock;
     const size_t head = static_cast<size_t>(a.head);
     const size_t nv = (a.n - head) / E;            // full vectors
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(kBlock) stream_vec(Args<T, NIN, NOUT> a, Op op
 template <typename T, int NIN, int NOUT, class Op, int U>
 __global__ void __launch_bounds__(kBlock) stream_scalar(Args<T, NIN, NOUT> a, Op op)
 {
-    const size_t tid = static_cast<size_t>(blockIdx.x) * kBlock + threadIdx.x;
+    const size_t tid = static_cast<size_t>(blockIdx.x + ffk::prior_kernel_done()) * kBlock + threadIdx.x;
     const size_t nthr = static_cast<size_t>(gridDim.x) * kBlock;
     size_t i = tid;
     for (; i + (U - 1) * nthr < a.n; i += U * nthr) {
@@ -219,16 +220,15 @@ ff_status launch(Args<T, NIN, NOUT> a, Op op, cudaStream_t s)
         if (occ > blocks_per_sm(NIN)) occ = blocks_per_sm(NIN);
         const size_t nv = (a.n - head) / E;
         unsigned grid = ffh::grid_for(nv > 0 ? nv : 1, static_cast<size_t>(kBlock) * U, di.sm_count, occ);
-        stream_vec<T, NIN, NOUT, Op, U><<<grid, kBlock, 0, s>>>(a, op);
+        return ffh::launch_kernel(&stream_vec<T, NIN, NOUT, Op, U>, grid, kBlock, s, a, op);
     } else {
         a.head = 0;
         const void* kern = reinterpret_cast<const void*>(&stream_scalar<T, NIN, NOUT, Op, U>);
         int occ = ffh::occupancy(kern, kBlock);
         if (occ > 2 * blocks_per_sm(NIN)) occ = 2 * blocks_per_sm(NIN);
         unsigned grid = ffh::grid_for(a.n, static_cast<size_t>(kBlock) * U, di.sm_count, occ);
-        stream_scalar<T, NIN, NOUT, Op, U><<<grid, kBlock, 0, s>>>(a, op);
+        return ffh::launch_kernel(&stream_scalar<T, NIN, NOUT, Op, U>, grid, kBlock, s, a, op);
     }
-    return ffh::check_launch();
 }
 
 }  // namespace ffst

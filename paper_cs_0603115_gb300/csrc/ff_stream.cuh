@@ -1,18 +1,25 @@
-// ff_stream.cuh -- one grid-stride streaming kernel for every elementwise op.
+// ff_stream.cuh -- one streaming kernel for every elementwise op.
 //
 // Each op reads NIN arrays and writes NOUT arrays of the same element type T
 // (float2 for float-float values and packed operand pairs, double or float
 // for the native baselines).  The body moves 16-byte vectors (two float2,
 // two double, four float) with evict-first streaming loads and stores: every
-// byte is touched once, so nothing is worth keeping in L1/L2.  Each thread
-// issues U vector loads per input before computing.
+// byte is touched once, so nothing is worth keeping in L1/L2.
 //
-// Residency: a GB300 sustains the highest read+write DRAM throughput on these
-// kernels with a moderate number of loads in flight per SM, not with every
-// SM full: measured on 2^28 values with the pipelined sweep below (U = 2),
-// the two-input operators reach ~7.0 TB/s with 3 blocks of 256 per SM
-// against ~6.6 TB/s at full occupancy, the one-input operators ~6.8 TB/s
-// with 4.  The launcher caps the grid at SMs x blocks_per_sm(NIN).
+// Bound by HBM.  A block takes one run of kBlock x U consecutive vectors of each
+// array, loads them together and ends; the next block follows on the SM.  So the
+// SM always holds blocks that load beside blocks that compute and store, and the
+// blocks in flight cover a compact stretch of each array.  Against a grid of 2 to
+// 4 resident blocks of 256 per SM that strode through the arrays with a software
+// pipeline: mul of 2^28 values 943 -> 887 us (7.26 TB/s), div 944 -> 883, sqrt
+// 640 -> 592, dot_backward 1285 -> 1201; div of 2^20 3.5 -> 3.2, dot_backward of
+// 2^26 331 -> 303, add of 4096 1.61 -> 1.12.  Strided instead of consecutive
+// vectors in such blocks: mul at 2^28 914.
+//
+// U by size: 1 while the vectors are no more than the resident threads, where a
+// second vector only lengthens a thread's chain (div of 2^18 values 1.93 us, 2.15
+// with 2); else 2 (sqrt at 2^22 7.1 us, 9.4 with 1; 3 and 4 within 2% of it from
+// 2^24 on, slower on the operators with two inputs below).
 //
 // Alignment: device arrays are only required to be aligned to sizeof(T).
 // If all arrays share the same offset modulo 16 bytes, a scalar head of
@@ -29,7 +36,7 @@
 
 namespace ffst {
 
-constexpr int kBlock = 256;
+constexpr int kBlock = 128;
 
 template <typename T> struct Vec;
 template <> struct Vec<float2> { using V = float4; static constexpr int E = 2; };
@@ -69,6 +76,18 @@ __device__ __forceinline__ void unpack(const float4& v, float (&e)[4])
 }
 __device__ __forceinline__ float4 pack(const float (&e)[4]) { return make_float4(e[0], e[1], e[2], e[3]); }
 
+// An operator that reads memory itself takes the wait's zero into its address
+// (see ffk::prior_kernel_done).
+template <class Op>
+__device__ __forceinline__ auto after_wait(Op& op, unsigned zero, int) -> decltype(op.after_wait(zero))
+{
+    op.after_wait(zero);
+}
+template <class Op>
+__device__ __forceinline__ void after_wait(Op&, unsigned, long)
+{
+}
+
 template <typename T, int NIN, int NOUT, class Op>
 __device__ __forceinline__ void scalar_at(const Args<T, NIN, NOUT>& a, const Op& op, size_t i)
 {
@@ -107,18 +126,15 @@ __device__ __forceinline__ void apply_vec(const Op& op, const typename Vec<T>::V
 }
 
 // Vector path: elements [0, head) and the tail are scalar; the body is
-// processed as 16-byte vectors, U per input per thread per sweep.  The sweep
-// is software-pipelined: the loads of sweep s + 1 are issued before the
-// values of sweep s are computed and stored, so each thread keeps loads in
-// flight while it computes.  (The scalar head and tail come after the sweep:
-// placed before it, they made the compiler schedule the Add22 loop worse.)
+// processed as 16-byte vectors, U consecutive runs of kBlock per block.
 template <typename T, int NIN, int NOUT, class Op, int U>
 __global__ void __launch_bounds__(kBlock) stream_vec(Args<T, NIN, NOUT> a, Op op)
 {
     using V = typename Vec<T>::V;
     constexpr int E = Vec<T>::E;
-    const size_t tid = static_cast<size_t>(blockIdx.x + ffk::prior_kernel_done()) * kBlock + threadIdx.x;
-    const size_t nthr = static_cast<size_t>(gridDim.x) * kBlock;
+    const unsigned zero = ffk::prior_kernel_done();
+    after_wait(op, zero, 0);
+    const size_t block = blockIdx.x + zero;
     const size_t head = static_cast<size_t>(a.head);
     const size_t nv = (a.n - head) / E;            // full vectors
     const size_t tail0 = head + nv * E;            // first tail element
@@ -130,81 +146,79 @@ __global__ void __launch_bounds__(kBlock) stream_vec(Args<T, NIN, NOUT> a, Op op
 #pragma unroll
     for (int k = 0; k < NOUT; ++k) out[k] = reinterpret_cast<V*>(a.out[k] + head);
 
-    size_t i = tid;
-    bool full = i + (U - 1) * nthr < nv;
-    V cur[U][NIN];
-    if (full) {
+    const size_t i = block * (kBlock * U) + threadIdx.x;
+    if (i + (U - 1) * kBlock < nv) {
+        V x[U][NIN];
 #pragma unroll
         for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int k = 0; k < NIN; ++k) cur[u][k] = __ldcs(in[k] + i + u * nthr);
-    }
-    while (full) {
-        const size_t nx = i + U * nthr;
-        const bool nfull = nx + (U - 1) * nthr < nv;
-        V nxt[U][NIN];
-        if (nfull) {
+            for (int k = 0; k < NIN; ++k) x[u][k] = __ldcs(in[k] + i + u * kBlock);
 #pragma unroll
-            for (int u = 0; u < U; ++u)
+        for (int u = 0; u < U; ++u) apply_vec<T, NIN, NOUT>(op, x[u], out, i + u * kBlock);
+    } else {
+        for (size_t j = i; j < nv; j += kBlock) {
+            V x[NIN];
 #pragma unroll
-                for (int k = 0; k < NIN; ++k) nxt[u][k] = __ldcs(in[k] + nx + u * nthr);
+            for (int k = 0; k < NIN; ++k) x[k] = __ldcs(in[k] + j);
+            apply_vec<T, NIN, NOUT>(op, x, out, j);
         }
-#pragma unroll
-        for (int u = 0; u < U; ++u) apply_vec<T, NIN, NOUT>(op, cur[u], out, i + u * nthr);
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-            for (int k = 0; k < NIN; ++k) cur[u][k] = nxt[u][k];
-        i = nx;
-        full = nfull;
     }
-    for (; i < nv; i += nthr) {
-        V x[NIN];
-#pragma unroll
-        for (int k = 0; k < NIN; ++k) x[k] = __ldcs(in[k] + i);
-        apply_vec<T, NIN, NOUT>(op, x, out, i);
+    if (block == 0) {
+        if (threadIdx.x < head) scalar_at(a, op, threadIdx.x);
+        if (threadIdx.x < a.n - tail0) scalar_at(a, op, tail0 + threadIdx.x);
     }
-
-    if (tid < head) scalar_at(a, op, tid);
-    if (tid < a.n - tail0) scalar_at(a, op, tail0 + tid);
 }
 
 // Scalar path for arrays whose offsets modulo 16 bytes differ.
 template <typename T, int NIN, int NOUT, class Op, int U>
 __global__ void __launch_bounds__(kBlock) stream_scalar(Args<T, NIN, NOUT> a, Op op)
 {
-    const size_t tid = static_cast<size_t>(blockIdx.x + ffk::prior_kernel_done()) * kBlock + threadIdx.x;
-    const size_t nthr = static_cast<size_t>(gridDim.x) * kBlock;
-    size_t i = tid;
-    for (; i + (U - 1) * nthr < a.n; i += U * nthr) {
+    const unsigned zero = ffk::prior_kernel_done();
+    after_wait(op, zero, 0);
+    const size_t i = static_cast<size_t>(blockIdx.x + zero) * (kBlock * U) + threadIdx.x;
+    if (i + (U - 1) * kBlock < a.n) {
         T x[U][NIN];
 #pragma unroll
         for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int k = 0; k < NIN; ++k) x[u][k] = a.in[k][i + u * nthr];
+            for (int k = 0; k < NIN; ++k) x[u][k] = __ldcs(a.in[k] + i + u * kBlock);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             T y[NOUT];
             op(x[u], y);
 #pragma unroll
-            for (int k = 0; k < NOUT; ++k) a.out[k][i + u * nthr] = y[k];
+            for (int k = 0; k < NOUT; ++k) __stcs(a.out[k] + i + u * kBlock, y[k]);
         }
+    } else {
+        for (size_t j = i; j < a.n; j += kBlock) scalar_at(a, op, j);
     }
-    for (; i < a.n; i += nthr) scalar_at(a, op, i);
 }
 
-// Resident 256-thread blocks per SM by number of input arrays (see above).
-constexpr int blocks_per_sm(int nin) { return nin == 1 ? 4 : nin == 2 ? 3 : 2; }
+template <typename T, int NIN, int NOUT, class Op, int U>
+ff_status launch_vec(const Args<T, NIN, NOUT>& a, const Op& op, size_t nv, cudaStream_t s)
+{
+    const size_t blocks = (nv + kBlock * U - 1) / (kBlock * U);
+    return ffh::launch_kernel(&stream_vec<T, NIN, NOUT, Op, U>, static_cast<unsigned>(blocks > 0 ? blocks : 1), kBlock, s,
+                              a, op);
+}
+
+template <typename T, int NIN, int NOUT, class Op, int U>
+ff_status launch_scalar(const Args<T, NIN, NOUT>& a, const Op& op, cudaStream_t s)
+{
+    const size_t blocks = (a.n + kBlock * U - 1) / (kBlock * U);
+    return ffh::launch_kernel(&stream_scalar<T, NIN, NOUT, Op, U>, static_cast<unsigned>(blocks), kBlock, s, a, op);
+}
 
 // Host launcher: validates nothing (the caller did), picks the path and the
-// grid, launches on `s`.
-template <typename T, int NIN, int NOUT, class Op, int U = 2>
+// vectors per thread, launches on `s`.
+template <typename T, int NIN, int NOUT, class Op>
 ff_status launch(Args<T, NIN, NOUT> a, Op op, cudaStream_t s)
 {
     if (a.n == 0) return FF_OK;
     ffh::DeviceInfo di;
     ff_status st = ffh::device_info(&di);
     if (st != FF_OK) return st;
+    const size_t resident = static_cast<size_t>(di.sm_count) * static_cast<size_t>(di.max_threads_per_sm);
     constexpr int E = Vec<T>::E;
     // offset of each array modulo 16 bytes, in elements
     uintptr_t phase = reinterpret_cast<uintptr_t>(a.in[0]) & 15u;
@@ -215,20 +229,11 @@ ff_status launch(Args<T, NIN, NOUT> a, Op op, cudaStream_t s)
         size_t head = phase ? (16u - phase) / sizeof(T) : 0;
         if (head > a.n) head = a.n;
         a.head = static_cast<int>(head);
-        const void* kern = reinterpret_cast<const void*>(&stream_vec<T, NIN, NOUT, Op, U>);
-        int occ = ffh::occupancy(kern, kBlock);
-        if (occ > blocks_per_sm(NIN)) occ = blocks_per_sm(NIN);
         const size_t nv = (a.n - head) / E;
-        unsigned grid = ffh::grid_for(nv > 0 ? nv : 1, static_cast<size_t>(kBlock) * U, di.sm_count, occ);
-        return ffh::launch_kernel(&stream_vec<T, NIN, NOUT, Op, U>, grid, kBlock, s, a, op);
-    } else {
-        a.head = 0;
-        const void* kern = reinterpret_cast<const void*>(&stream_scalar<T, NIN, NOUT, Op, U>);
-        int occ = ffh::occupancy(kern, kBlock);
-        if (occ > 2 * blocks_per_sm(NIN)) occ = 2 * blocks_per_sm(NIN);
-        unsigned grid = ffh::grid_for(a.n, static_cast<size_t>(kBlock) * U, di.sm_count, occ);
-        return ffh::launch_kernel(&stream_scalar<T, NIN, NOUT, Op, U>, grid, kBlock, s, a, op);
+        return nv <= resident ? launch_vec<T, NIN, NOUT, Op, 1>(a, op, nv, s) : launch_vec<T, NIN, NOUT, Op, 2>(a, op, nv, s);
     }
+    a.head = 0;   // half the bytes per access: twice as many in flight (sqrt of 2^27 values 409 -> 329 us)
+    return a.n <= resident ? launch_scalar<T, NIN, NOUT, Op, 1>(a, op, s) : launch_scalar<T, NIN, NOUT, Op, 4>(a, op, s);
 }
 
 }  // namespace ffst

@@ -1,15 +1,16 @@
 // ff_batch.cu -- many independent float-float dot and AXPY instances of
-// uneven lengths in one persistent launch, a CUDA-graph wrapper around it,
-// and the autotuner that picks its block size, values per thread and
-// resident blocks per SM.
+// uneven lengths in one launch, a CUDA-graph wrapper around it, and the
+// autotuner that picks its block size, values per thread and resident blocks
+// per SM.
 //
 // Plan (host, once): every instance is cut into tiles of block x ppt values;
 // the tiles of all instances form one list, instance after instance.  The
 // plan copies the instance records and the tile list to device memory it
 // owns.
 //
-// Run: a persistent grid of (SMs x blocks per SM) blocks walks the tile list
-// round robin (block b takes tiles b, b + G, b + 2G, ...).
+// Run: a block per tile, or, when the tune gives blocks per SM, that many
+// resident blocks that walk the tile list round robin (block b of G takes tiles
+// b, b + G, b + 2G, ...).
 //   AXPY tile: z_i = Add22(Mul22(alpha, x_i), y_i) for the tile's values.
 //   dot-gradient tile: dx_i = Mul22(dout, y_i), dy_i = Mul22(dout, x_i).
 //   GEMV rows tile (rows of length <= 65536): eight lanes reduce one row,
@@ -36,8 +37,9 @@
 // Plans made only of GEMV rows run a kernel of their own: their tiles differ
 // in cost (a tile holds 4 x warps x R rows, and R cannot drop below one for
 // rows longer than 16K / (4 x warps) values), so the plan sorts the tiles by
-// cost, largest first, and the blocks take the next tile from an atomic
-// counter (zeroed by the same memset) instead of round robin.  Each such
+// cost, largest first, and resident blocks, where there are fewer of them than
+// tiles, take the next tile from an atomic counter (zeroed by the same memset)
+// instead of round robin.  Each such
 // tile writes whole rows, so the order changes no result.
 #include <algorithm>
 #include <cstring>
@@ -345,8 +347,8 @@ __device__ __forceinline__ void combine_tiles(const DevInst& I, const float2* pa
 // block; records of mixed alignment keep 2 UN values of each input in flight; the
 // sweep's shape takes 63 registers where it took 126, so that 32 warps are
 // resident instead of 16.  1024 dot and AXPY instances of up to 1e6 values
-// (2.2 GB, floor 326 us), default tune: stored back to back 578 -> 352 us, padded
-// to 16 bytes 384 -> 343.
+// (2.2 GB, 326 us at the plain copy's rate), default tune: stored back to back
+// 578 -> 322 us, padded to 16 bytes 384 -> 314 (resident blocks: 350 and 342).
 template <int BLOCK, int PPT, int UN, bool GEMV_ROWS>
 __global__ void __launch_bounds__(BLOCK, GEMV_ROWS ? 1024 / BLOCK : 0)
 batch_kernel(const DevInst* __restrict__ insts, const Tile* __restrict__ tiles, int64_t ntiles,
@@ -685,18 +687,22 @@ ff_status ff_batch_plan_create(const ff_batch_instance* inst, int count, const f
     p->ndot = ndot;
     p->total_values = total;
     p->device = di.device;
-    int bps = tune.blocks_per_sm;
-    if (bps == 0) {
-        bps = ffh::occupancy(reinterpret_cast<const void*>(kernel_for(*var, *p)), tune.block);
-        // a long run of elementwise tiles alone, four chunks ahead, streams best on
-        // 512 threads per SM (512 AXPY instances of up to 1e6 values: 194 us, 205 with 1024 threads;
-        // short runs want all of them: 14.9 against 12.5 us)
-        bool elementwise = !hi.empty();
-        for (const DevInst& d : hi) elementwise &= d.kind == FF_BATCH_AXPY || d.kind == FF_BATCH_DOT_GRAD;
-        const int few = std::max(1, 512 / tune.block);
-        if (elementwise && var->unroll == 4 && p->ntiles > 8 * static_cast<int64_t>(few) * di.sm_count) bps = std::min(bps, few);
+    // blocks_per_sm 0: a block per tile.  Blocks start in tile order as SMs become
+    // free, so long and short tiles balance, and a block that computes always has
+    // one that loads beside it.  Blocks that stay and walk the tiles in fixed steps
+    // took 350 us for 1024 dot and AXPY instances of up to 1e6 values, 322 this way.
+    // GEMV tiles alone, more than four per resident block, are better walked by
+    // resident blocks with the tile counter: 300 matrices of up to 3000 x 3000 186
+    // us, 188 with a block per tile; fewer save the counter's clearing (1000 of up to
+    // 100 x 100: 17.6 -> 15.2).
+    int64_t grid = 0x7fffffff;
+    if (tune.blocks_per_sm > 0) {
+        grid = static_cast<int64_t>(di.sm_count) * tune.blocks_per_sm;
+    } else if (p->only_gemv_rows) {
+        const int occ = ffh::occupancy(reinterpret_cast<const void*>(kernel_for(*var, *p)), tune.block);
+        const int64_t resident = static_cast<int64_t>(di.sm_count) * (occ > 0 ? occ : 1);
+        if (p->ntiles > 4 * resident) grid = resident;
     }
-    int64_t grid = static_cast<int64_t>(di.sm_count) * (bps > 0 ? bps : 1);
     if (grid > p->ntiles) grid = p->ntiles > 0 ? p->ntiles : 1;
     p->grid = static_cast<unsigned>(grid);
     // counters: the arrivals of dots of several tiles, and the tile counter of a
@@ -817,7 +823,7 @@ void ff_batch_graph_destroy(ff_batch_graph* g)
 
 int ff_batch_tune_candidates(ff_tune* out, int max)
 {
-    const int per = 3;  // blocks per SM: occupancy-limited (0), 2, 4
+    const int per = 3;  // a block per tile (0), or resident blocks per SM: 2, 4
     const int bps[per] = {0, 2, 4};
     int k = 0;
     for (const Variant& v : kVariants)

@@ -689,20 +689,31 @@ gemv_dA_small_kernel(const float2* __restrict__ dY, int64_t m, int64_t lddy, con
 constexpr int kDAPair = 12;
 constexpr int kDAMaxSmallK = 20;
 
-// Grid of one wave of resident blocks (rounded down so that every block is
-// resident at once), block rows of whole steps.
+// Grid: as many block rows as fill 1 to 8 waves of resident blocks, whichever
+// takes the fewest rows in turn, a wave's start counted as four rows.  One wave
+// alone leaves up to a block row of slots empty: at 32768 columns and three
+// blocks per SM 384 of 456 slots, k = 20 15.9 ms, 13.4 in two waves.
 template <int KT, int E>
 ff_status launch_dA(const float2* dY, int64_t m, int64_t lddy, const float2* X, int64_t n, int64_t ldx, float2* dA,
                     int64_t ldda, int sm_count, cudaStream_t s)
 {
     const int64_t col_blocks = (n / E + kGBlock - 1) / kGBlock;
     const int occ = ffh::occupancy(reinterpret_cast<const void*>(&gemv_dA_small_kernel<KT, E>), kGBlock);
-    int64_t gy = static_cast<int64_t>(sm_count) * (occ > 0 ? occ : 1) / col_blocks;
+    const int64_t slots = static_cast<int64_t>(sm_count) * (occ > 0 ? occ : 1);
     constexpr int64_t RS = 4 / E;
-    if (gy > (m + RS - 1) / RS) gy = (m + RS - 1) / RS;
-    if (gy > 65535) gy = 65535;
-    if (gy < 1) gy = 1;
-    const int64_t rpb = ((m + gy - 1) / gy + RS - 1) / RS * RS;
+    int64_t rpb = 0, least = 0;
+    for (int w = 1; w <= 8; ++w) {
+        int64_t gy = w * slots / col_blocks;
+        if (gy > (m + RS - 1) / RS) gy = (m + RS - 1) / RS;
+        if (gy > 65535) gy = 65535;
+        if (gy < 1) gy = 1;
+        const int64_t rows = ((m + gy - 1) / gy + RS - 1) / RS * RS;
+        const int64_t waves = (col_blocks * ((m + rows - 1) / rows) + slots - 1) / slots;
+        if (w == 1 || waves * (rows + 4) < least) {
+            rpb = rows;
+            least = waves * (rows + 4);
+        }
+    }
     const dim3 grid(static_cast<unsigned>(col_blocks), static_cast<unsigned>((m + rpb - 1) / rpb));
     return ffh::launch_kernel(&gemv_dA_small_kernel<KT, E>, grid, kGBlock, s, dY, m, lddy, X, n, ldx, dA, ldda, rpb);
 }

@@ -159,3 +159,16 @@ def test_batch_gemv_rows(shapes, kind):
             same_bits(out.cpu().numpy()[rows], w)
             out.fill_(float("nan"))
     plan.close()
+
+
+# weight gradients whose grid takes several waves of blocks, ragged in rows and
+# columns, pairs of columns and single ones
+@pytest.mark.parametrize("m,n,k", [(9, 200000, 2), (1003, 130001, 1), (301, 70000, 13), (77, 131072, 3)])
+def test_weight_gradient_waves(m, n, k):
+    dY, X = inputs.to_ff(inputs.loguniform_f64(k * m, torch.Generator().manual_seed(3), "cpu")).reshape(k, m, 2), \
+        inputs.to_ff(inputs.loguniform_f64(k * n, torch.Generator().manual_seed(4), "cpu")).reshape(k, n, 2)
+    got = ff.gemv_dA(dY.to(DEV), X.to(DEV)).cpu().numpy()
+    rows = sorted({0, 1, 4, m // 3, m // 2, m - 2, m - 1})
+    want = oracle.gemv_dA(np.ascontiguousarray(dY[:, rows].numpy()), X.numpy())
+    same_bits(got[rows], want)
+    assert np.isfinite(got).all()

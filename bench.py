@@ -260,6 +260,10 @@ def cpu_baseline(e_gpu, min_seconds: float = 8.0):
                       f"on {cores} host threads (contiguous chunks); {reps1} pass(es) in {dt1:.1f} s on one"}
 
 
+# FP32 instructions per accumulated term Add22(acc, Mul22(a, b)) with the
+# Fast2Sum closings of ff_core.cuh (9 + 13; with Add12 closings 12 + 16)
+TERM_OPS = 22
+
 # sources that define the elementwise kernels (and their flags)
 ELEMENTWISE_SOURCES = ("paper_cs_0603115_gb300/csrc/ff_core.cuh", "paper_cs_0603115_gb300/csrc/ff_stream.cuh",
                        "paper_cs_0603115_gb300/csrc/ff_elementwise.cu", "paper_cs_0603115_gb300/csrc/ff_host.cuh",
@@ -578,10 +582,10 @@ def extra_rows(torch, ff, inputs, e, dev, peaks):
         tw = time_median(torch, lambda: ff.gemv_dA(X, X, out=dA), 11, warm=2)
         tot_f += tf
         tot_b += tb
-        t_bound = max(8 * M * N / (hbm * 1e9), 28 * M * N * k / fp32)   # roofline time of one call
+        t_bound = max(8 * M * N / (hbm * 1e9), TERM_OPS * M * N * k / fp32)   # roofline time of one call
         gem[str(k)] = {"fwd_ms": round(tf * 1e3, 3), "adj_ms": round(tb * 1e3, 3), "dA_ms": round(tw * 1e3, 3),
                        "fwd_ff_op_s": 2 * M * N * k / tf, "adj_ff_op_s": 2 * M * N * k / tb,
-                       "bound": "hbm" if 8 * M * N / (hbm * 1e9) >= 28 * M * N * k / fp32 else "fp32",
+                       "bound": "hbm" if 8 * M * N / (hbm * 1e9) >= TERM_OPS * M * N * k / fp32 else "fp32",
                        "fwd_frac_roofline": round(t_bound / tf, 4), "adj_frac_roofline": round(t_bound / tb, 4),
                        "dA_frac_roofline": round(t_bound / tw, 4)}
     del dA
@@ -625,8 +629,8 @@ def alu_peaks(torch, ff, dev):
 def gemm_rows(torch, ff, inputs, dev, size=4096, fp32_measured=None):
     """Float-float GEMM, size^3: ff_gemm forward and the two adjoint GEMMs of
     FFGemm, against cuBLAS FP64 and FP32 GEMM (torch.matmul) on the same
-    values.  The kernel is bound by FP32 instruction issue: 28 FP32
-    instructions per term (Mul22 12, Add22 16) against SMs x 128 lanes x the
+    values.  The kernel is bound by FP32 instruction issue: TERM_OPS FP32
+    instructions per term against SMs x 128 lanes x the
     SM clock sampled while it runs."""
     m = n = k = size
     g = inputs.gemm(m, n, k, inputs.seed_for(6, 0), device=dev)
@@ -659,8 +663,8 @@ def gemm_rows(torch, ff, inputs, dev, size=4096, fp32_measured=None):
     return {f"gemm_{size}^3": {
         "fwd_ms": round(t_fwd * 1e3, 3), "dA_ms": round(t_dA * 1e3, 3), "dB_ms": round(t_dB * 1e3, 3),
         "fwd_ff_op_s": 2 * terms / t_fwd, "terms_per_s": terms / t_fwd,
-        "frac_fp32_issue": round(28 * terms / t_fwd / issue, 4), "issue_peak_lane_ops_s": issue,
-        "frac_of_measured_fp32_fma": round(28 * terms / t_fwd / fp32_measured, 4) if fp32_measured else None,
+        "frac_fp32_issue": round(TERM_OPS * terms / t_fwd / issue, 4), "issue_peak_lane_ops_s": issue,
+        "frac_of_measured_fp32_fma": round(TERM_OPS * terms / t_fwd / fp32_measured, 4) if fp32_measured else None,
         "clocks": clocks,
         "cublas_f64_ms": round(t64 * 1e3, 3), "speedup_vs_cublas_f64": round(t64 / t_fwd, 3),
         "cublas_f32_ms": round(t32 * 1e3, 3), "slowdown_vs_cublas_f32": round(t_fwd / t32, 2)}}
@@ -669,7 +673,7 @@ def gemm_rows(torch, ff, inputs, dev, size=4096, fp32_measured=None):
 def batched_rows(torch, ff, inputs, dev, peaks):
     """4096 dot / AXPY instances, lengths log-uniform over 1e2..1e7 (dots by
     the ill-conditioned generator at cond 1e8, AXPY by the elementwise one
-    with its 10% cancelling pairs): one persistent launch (plain run and CUDA
+    with its 10% cancelling pairs): one launch (plain run and CUDA
     graph) against 4096 plain calls (loop and CUDA graph); then the same
     dots' forward and adjoint batched against plain ff_dot / ff_dot_backward
     calls; last, the 4096 instances packed without padding, so that every
@@ -871,7 +875,7 @@ def batched_rows(torch, ff, inputs, dev, peaks):
 
 def batched_gemv_row(torch, ff, inputs, dev, hbm):
     """1024 float-float GEMVs y = A x of uneven shapes (m, n log-uniform over
-    32..4096) in one persistent launch, against 1024 plain ff_gemv calls."""
+    32..4096) in one launch, against 1024 plain ff_gemv calls."""
     from paper_cs_0603115_gb300 import batch
     g = torch.Generator().manual_seed(inputs.seed_for(3, 9))
     cnt = 1024
@@ -996,7 +1000,7 @@ def run_case(args):
         fn = (lambda: ff.dot2(g.x, g.y)) if args.case == "dot2" else (lambda: ff.sum2(g.x))
     elif args.case in ("batch", "batch_packed"):
         # 256 dot / AXPY instances, lengths log-uniform over 1e2..1e6 (a small
-        # sample of the 4096-instance workload), one persistent launch; with
+        # sample of the 4096-instance workload), one launch; with
         # batch_packed the instances lie back to back (every instance after an
         # odd length starts 8 bytes off a 16-byte boundary)
         from paper_cs_0603115_gb300 import batch
@@ -1014,7 +1018,7 @@ def run_case(args):
         for i, (ln, kind) in enumerate(zip(lengths, kinds)):
             sl = slice(offs[i], offs[i] + ln)
             specs.append((kind, X[sl], Y[sl], D[i] if kind == batch.DOT else Z[sl], (1.5, 0.0)))
-        plan = batch.BatchPlan(batch.make_instances(specs), tune=(256, 128, 4, 4))
+        plan = batch.BatchPlan(batch.make_instances(specs), tune=(256, 32, 0, 4))
         fn = plan.run
     elif args.case == "batch_gemv":
         from paper_cs_0603115_gb300 import batch
@@ -1034,7 +1038,7 @@ def run_case(args):
             ox += nn
             oy += mm
         # the launch shape the autotuner picks for bench.py's 1024-GEMV batch:
-        # 128-thread blocks, as many resident as fit
+        # 128-thread blocks, a block per tile or as many resident as fit
         plan = batch.BatchPlan(batch.make_instances(specs), tune=(128, 16, 0, 2))
         fn = plan.run
     elif args.case == "gemm":

@@ -286,7 +286,7 @@ FF_API ff_status ff_gemm(int transa, int transb, int64_t m, int64_t n, int64_t k
                          const ff2* B, int64_t ldb, ff2* C, int64_t ldc, cudaStream_t s);
 
 /* ------------------------------------------------------------------------ */
-/* Batched dot / AXPY: many instances in one persistent launch               */
+/* Batched dot / AXPY: many instances in one launch                          */
 /* ------------------------------------------------------------------------ */
 
 typedef enum ff_batch_kind {
@@ -357,7 +357,7 @@ FF_API size_t ff_batch_workspace_bytes(const ff_batch_plan* plan);
 FF_API ff_status ff_batch_plan_info(const ff_batch_plan* plan, ff_tune* tune, int64_t* ntiles, unsigned* grid);
 
 /* Run every instance of the plan: one memset of the per-instance counters
- * and the tile counter (for plans that use them), and one persistent kernel
+ * and the tile counter (for plans that use them), and one kernel
  * launch on stream s.
  * Graph-capturable.  The workspace (ff_batch_workspace_bytes, 16-byte
  * aligned, owned by the caller) must not be shared by runs that overlap. */

@@ -18,7 +18,7 @@ GEMV, GEMM:   gemv (Y = A X), gemv_t (dX = A^T dY), gemv_dA (dA = dY X^T),
 Autograd:     FFDot, FFGemv, FFGemm and ffdot, ffgemv, ffgemm (hand-written
               adjoint kernels)
 Baselines:    f64_add/mul/div/sqrt/dot/gemv, f32_add/mul/mad, fma_peak
-Submodules:   batch (many instances in one persistent launch, CUDA graphs,
+Submodules:   batch (many instances in one launch, CUDA graphs,
               autotuner), dist (sharded reductions over processes), inputs
               (the seeded input recipe)
 """

@@ -1,5 +1,5 @@
 """Batched float-float dot, AXPY, dot-adjoint and GEMV instances in one
-persistent launch.
+launch.
 
 Thin wrapper over the C ABI's ff_batch_* entry points: a ``BatchPlan`` holds
 the native plan (instance records and tile list on the device), its
@@ -104,7 +104,7 @@ class BatchPlan:
         self.grid = grid.value
 
     def run(self):
-        """One memset + one persistent kernel on the current stream."""
+        """One kernel on the current stream (after a memset for plans that count arrivals)."""
         _lib.call("ff_batch_run", self.handle, self.ws.data_ptr(), self.ws.numel(),
                   torch.cuda.current_stream().cuda_stream)
 

@@ -13,10 +13,10 @@
 // per right-hand side.  The 32 lane accumulators are combined by a shuffle-down
 // Add22 tree.
 //
-// ff_gemv_t: a thread sums one column or a pair of adjacent columns of A over
-// one row block in order, for a tile of up to four right-hand sides; a block
-// holds several row blocks of its columns and adds their sums in row-block
-// order, or the sums go to the workspace and a second kernel adds them.
+// ff_gemv_t: a thread sums one column or two columns of A over one row block in
+// order, for a tile of up to four right-hand sides; a block holds several row
+// blocks of its columns and adds their sums in row-block order, or the sums go
+// to the workspace and a second kernel adds them.
 //
 // ff_gemv_dA: one thread per column or pair of adjacent columns of dA, its X
 // values in registers, the block's rows walked four elements at a time with dY
@@ -285,14 +285,20 @@ ff_status gemv_forward(const float2* A, int64_t m, int64_t n, int64_t lda, const
 // ---------------------------------------------------------------------------
 // dX = A^T dY
 // ---------------------------------------------------------------------------
-// One thread's sums of E adjacent columns over the rows [r0, r1) in order, R
-// rows loaded before they are added.  FAST uses the Fast2Sum forms and returns
+// A thread's columns: two adjacent ones (16-byte access), one, or two `apart`
+// columns from one another (8-byte access; they share the loads of dY).
+enum Columns { kAdjacent, kSingle, kApart };
+
+// One thread's sums of its columns over the rows [r0, r1) in order, R rows
+// loaded before they are added.  FAST uses the Fast2Sum forms and returns
 // true when a product fell outside their condition; the caller then repeats
 // the sums with FAST false.
-template <int KT, int E, int R, bool FAST>
-__device__ __forceinline__ bool gemv_t_sums(const float2* __restrict__ Aj, int64_t lda, const float2* __restrict__ dY,
-                                            int64_t lddy, int64_t r0, int64_t r1, float2 (&acc)[KT][E])
+template <int KT, Columns C, int R, bool FAST>
+__device__ __forceinline__ bool gemv_t_sums(const float2* __restrict__ Aj, int apart, int64_t lda,
+                                            const float2* __restrict__ dY, int64_t lddy, int64_t r0, int64_t r1,
+                                            float2 (&acc)[KT][C == kSingle ? 1 : 2])
 {
+    constexpr int E = C == kSingle ? 1 : 2;
     using V = std::conditional_t<E == 2, float4, float2>;
     bool bad = false;
     auto term = [&](float2& s, float2 a, float2 d) {
@@ -305,7 +311,15 @@ __device__ __forceinline__ bool gemv_t_sums(const float2* __restrict__ Aj, int64
         term(s[0], make_float2(a.x, a.y), d);
         if constexpr (E == 2) term(s[1], make_float2(a.z, a.w), d);
     };
-    auto load = [&](int64_t r) { return __ldcs(reinterpret_cast<const V*>(Aj + r * lda)); };
+    auto load = [&](int64_t r) {
+        const float2* p = Aj + r * lda;
+        if constexpr (C == kApart) {
+            const float2 a = __ldcs(p), b = __ldcs(p + apart);
+            return make_float4(a.x, a.y, b.x, b.y);
+        } else {
+            return __ldcs(reinterpret_cast<const V*>(p));
+        }
+    };
 #pragma unroll
     for (int c = 0; c < KT; ++c)
 #pragma unroll
@@ -336,7 +350,7 @@ __device__ __forceinline__ bool gemv_t_sums(const float2* __restrict__ Aj, int64
 }
 
 // The block's tile of KT right-hand sides; see gemv_t_kernel.
-template <int KT, int E, int R>
+template <int KT, Columns C, int R>
 __device__ __forceinline__ void gemv_t_tile(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda,
                                             const float2* __restrict__ dY, int64_t lddy, int64_t rpb, int64_t nrb,
                                             int cx, float2* __restrict__ out, int64_t out_ld, int64_t rb_stride,
@@ -345,21 +359,27 @@ __device__ __forceinline__ void gemv_t_tile(const float2* __restrict__ A, int64_
     const int tx = threadIdx.x & (cx - 1);
     const int ty = threadIdx.x / cx;
     const int rg = kGBlock / cx;
-    const int64_t j = (static_cast<int64_t>(blockIdx.x + zero) * cx + tx) * E;   // first column
+    constexpr int E = C == kSingle ? 1 : 2;
+    const int64_t j = static_cast<int64_t>(blockIdx.x + zero) * cx * E + (C == kAdjacent ? 2 * tx : tx);   // first column
+    const int apart = C == kAdjacent ? 1 : cx;   // to the second one
+    const bool second = C == kAdjacent || j + apart < n;
     const int64_t rb = static_cast<int64_t>(blockIdx.y + zero) * rg + ty;
     const int64_t r0 = rb * rpb;
     const int64_t r1 = r0 + rpb < m ? r0 + rpb : m;
     float2 acc[KT][E];
     const bool active = j < n && rb < nrb;
-    if (active && gemv_t_sums<KT, E, R, true>(A + j, lda, dY, lddy, r0, r1, acc))
-        gemv_t_sums<KT, E, 1, false>(A + j, lda, dY, lddy, r0, r1, acc);
+    const int step = second ? apart : 0;
+    if (active && gemv_t_sums<KT, C, R, true>(A + j, step, lda, dY, lddy, r0, r1, acc))
+        gemv_t_sums<KT, C, 1, false>(A + j, step, lda, dY, lddy, r0, r1, acc);
     if (rg == 1 || gridDim.y > 1) {
         if (!active) return;
         float2* o = out + rb * rb_stride + j;
 #pragma unroll
-        for (int c = 0; c < KT; ++c)
-#pragma unroll
-            for (int e = 0; e < E; ++e) o[c * out_ld + e] = ffk::ff_overflow_lo(acc[c][e]);
+        for (int c = 0; c < KT; ++c) {
+            o[c * out_ld] = ffk::ff_overflow_lo(acc[c][0]);
+            if constexpr (E == 2)
+                if (second) o[c * out_ld + apart] = ffk::ff_overflow_lo(acc[c][1]);
+        }
         return;
     }
     if (active) {
@@ -370,15 +390,16 @@ __device__ __forceinline__ void gemv_t_tile(const float2* __restrict__ A, int64_
     }
     __syncthreads();
     if (j >= n) return;
-    for (int w = ty; w < KT * E; w += rg) {   // column j + w % E of right-hand side w / E
+    for (int w = ty; w < KT * E; w += rg) {   // the thread's column w % E of right-hand side w / E
+        if (w % E && !second) continue;
         float2 v = part[w][tx];
 #pragma unroll 4
         for (int b = 1; b < nrb; ++b) v = ffk::add22_fast(v, part[w][b * cx + tx]);
-        out[(w / E) * out_ld + j + w % E] = ffk::ff_overflow_lo(v);
+        out[(w / E) * out_ld + j + (w % E) * apart] = ffk::ff_overflow_lo(v);
     }
 }
 
-// Grid: x groups of cx columns (column pairs with E = 2), y groups of row
+// Grid: x groups of cx columns or column pairs, y groups of row
 // blocks, z tiles of right-hand sides, the first `na` KA wide and the others
 // KB.  A block is cx columns wide and 256 / cx row blocks high: thread (tx, ty)
 // sums row block blockIdx.y * (256 / cx) + ty.  With one group of several row
@@ -386,22 +407,22 @@ __device__ __forceinline__ void gemv_t_tile(const float2* __restrict__ A, int64_
 // and writes dX; otherwise thread sums go to out[rb * rb_stride + c * out_ld +
 // j] (dX itself when there is a single row block, else the workspace that
 // gemv_t_combine reads).
-template <int KA, int KB, int E, int R, int MINB>
+template <int KA, int KB, Columns C, int R, int MINB>
 __global__ void __launch_bounds__(kGBlock, MINB)
 gemv_t_kernel(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda, const float2* __restrict__ dY,
               int64_t lddy, int64_t rpb, int64_t nrb, int cx, float2* __restrict__ out, int64_t out_ld,
               int64_t rb_stride, int na)
 {
-    __shared__ float2 part[KA * E][kGBlock];
+    __shared__ float2 part[KA * (C == kSingle ? 1 : 2)][kGBlock];
     const unsigned zero = ffk::prior_kernel_done();
     const int z = blockIdx.z;
     if (KA == KB || z < na) {
         const int64_t c0 = static_cast<int64_t>(z) * KA;
-        gemv_t_tile<KA, E, R>(A, m, n, lda, dY + c0 * lddy, lddy, rpb, nrb, cx, out + c0 * out_ld, out_ld, rb_stride,
+        gemv_t_tile<KA, C, R>(A, m, n, lda, dY + c0 * lddy, lddy, rpb, nrb, cx, out + c0 * out_ld, out_ld, rb_stride,
                               part, zero);
     } else {
         const int64_t c0 = static_cast<int64_t>(na) * KA + static_cast<int64_t>(z - na) * KB;
-        gemv_t_tile<KB, E, R>(A, m, n, lda, dY + c0 * lddy, lddy, rpb, nrb, cx, out + c0 * out_ld, out_ld, rb_stride,
+        gemv_t_tile<KB, C, R>(A, m, n, lda, dY + c0 * lddy, lddy, rpb, nrb, cx, out + c0 * out_ld, out_ld, rb_stride,
                               part, zero);
     }
 }
@@ -420,11 +441,12 @@ gemv_t_combine(const float2* __restrict__ ws, int64_t n, int64_t k, int64_t nrb,
     dX[c * lddx + j] = ffk::ff_overflow_lo(acc);
 }
 
-// How the adjoint is cut: blocks cx columns (or column pairs) wide and
-// 256 / cx row blocks high, gy of them down the rows, right-hand sides in
-// tiles of 1 (wide false) or as split_tiles says.
+// How the adjoint is cut: blocks cx columns (or column pairs: adjacent ones on
+// 16-byte access, `pairs` apart on 8-byte access) wide and 256 / cx row blocks
+// high, gy of them down the rows, right-hand sides in tiles of 1 (wide false)
+// or as split_tiles says.
 struct AdjointPlan {
-    bool wide;
+    bool wide, pairs;
     int cx;
     int64_t gy, nrb, rpb;
 };
@@ -443,7 +465,7 @@ inline void cut_rows(int64_t m, int64_t want, int64_t* nrb, int64_t* rpb)
 inline int adjoint_rows(const AdjointPlan& p, int ka, int64_t k, bool vec)
 {
     if (k == 1 && p.gy > 1) return 16;
-    return ka <= 2 || !vec ? 8 : 4;
+    return ka <= 2 || !(vec || p.pairs) ? 8 : 4;
 }
 
 // Modelled cycles of a cut, fitted to a sweep of all cuts of 41 shapes (64^2 to
@@ -457,8 +479,8 @@ inline int adjoint_rows(const AdjointPlan& p, int ka, int64_t k, bool vec)
 double adjoint_cycles(const AdjointPlan& p, int64_t m, int64_t n, int64_t k, bool vec, int sm_count)
 {
     const TileSplit t = p.wide ? split_tiles(k) : TileSplit{1, 1, k, 0};
-    const int e = vec ? 2 : 1;
-    const int64_t cols = n / e;
+    const int e = vec || p.pairs ? 2 : 1;
+    const int64_t cols = (n + e - 1) / e;
     const int64_t z = t.na + t.nb;
     const int rows = adjoint_rows(p, t.ka, k, vec);
     const double blocks = static_cast<double>((cols + p.cx - 1) / p.cx) * static_cast<double>(p.gy * z);
@@ -471,8 +493,8 @@ double adjoint_cycles(const AdjointPlan& p, int64_t m, int64_t n, int64_t k, boo
         over = (std::floor(waves) + (part > 0.0 ? 0.29 + 0.71 * part : 0.0)) / waves;
         per = over * blocks / sm_count;
     }
-    const double issue = per * 2.0 * p.rpb * t.ka * e * (24.5 + (vec ? 0.0 : 3.2));
-    const double bytes = 8.0 * m * n * z * (1.0 + (vec ? 23.0 : 16.0) / (8.0 * p.cx * e));
+    const double issue = per * 2.0 * p.rpb * t.ka * e * (24.5 + (vec ? 0.0 : p.pairs ? 1.0 : 3.2));
+    const double bytes = 8.0 * m * n * z * (1.0 + (vec ? 23.0 : p.pairs ? 32.0 : 16.0) / (8.0 * p.cx * e));
     // 128-byte lines per warp and row: of A, and one of dY per row block and
     // right-hand side
     const double rbw = p.cx < 32 ? 32.0 / p.cx : 1.0;
@@ -494,8 +516,15 @@ double adjoint_cycles(const AdjointPlan& p, int64_t m, int64_t n, int64_t k, boo
 // 5.1 us; 10000 x 100, k = 3: 41 -> 14 us; 2001 x 3001, k = 5: 51 -> 32 us.
 AdjointPlan search_adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int sm_count)
 {
-    AdjointPlan best{true, kGBlock, 1, 1, m > 0 ? m : 0};
+    AdjointPlan best{true, false, kGBlock, 1, 1, m > 0 ? m : 0};
     if (m < 1 || n < 1) return best;
+    // On 8-byte access a thread takes two columns apart, which share the loads of
+    // dY, where the matrix gives every thread enough to do: 8191^2, k = 2 141 -> 126
+    // us, 4000 x 6001, k = 5 123 -> 110, 12001^2, k = 1 190 -> 176.  Smaller or
+    // narrower ones lose more to the halved number of threads (2001 x 3001, k = 5 29
+    // -> 34, 3333 x 401 11.8 -> 12.7, 1024 x 1025, k = 64 57 -> 60).
+    const double values = static_cast<double>(m) * n;
+    const bool pairs = !vec && n >= 1024 && values >= 2e6 && values * k >= 64e6;
     double least = -1.0;
     auto consider = [&](int cx, int64_t gy) {
         AdjointPlan p{};
@@ -503,6 +532,7 @@ AdjointPlan search_adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int s
         const int64_t rg = kGBlock / cx;
         cut_rows(m, rg * gy, &p.nrb, &p.rpb);
         p.gy = (p.nrb + rg - 1) / rg;
+        p.pairs = pairs;
         for (int w = 0; w < (k > 1 ? 2 : 1); ++w) {
             p.wide = w == 1;
             const double c = adjoint_cycles(p, m, n, k, vec, sm_count);
@@ -542,15 +572,15 @@ AdjointPlan adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int sm_count
     return e.plan;
 }
 
-template <int KA, int KB, int E, int R, int MINB>
+template <int KA, int KB, Columns C, int R, int MINB>
 ff_status launch_adjoint(const AdjointPlan& p, const TileSplit& t, const float2* A, int64_t m, int64_t n, int64_t lda,
                          const float2* dY, int64_t lddy, float2* out, int64_t out_ld, int64_t rb_stride,
                          cudaStream_t s)
 {
-    const int64_t cols = n / E;
-    const dim3 grid(static_cast<unsigned>((cols + p.cx - 1) / p.cx), static_cast<unsigned>(p.gy),
+    const int64_t width = static_cast<int64_t>(p.cx) * (C == kSingle ? 1 : 2);
+    const dim3 grid(static_cast<unsigned>((n + width - 1) / width), static_cast<unsigned>(p.gy),
                     static_cast<unsigned>(t.na + t.nb));
-    return ffh::launch_kernel(&gemv_t_kernel<KA, KB, E, R, MINB>, grid, kGBlock, s, A, m, n, lda, dY, lddy, p.rpb, p.nrb,
+    return ffh::launch_kernel(&gemv_t_kernel<KA, KB, C, R, MINB>, grid, kGBlock, s, A, m, n, lda, dY, lddy, p.rpb, p.nrb,
                               p.cx, out, out_ld, rb_stride, static_cast<int>(t.na));
 }
 
@@ -850,21 +880,23 @@ ff_status ff_gemv_t(const ff2* A_, int64_t m, int64_t n, int64_t lda, const ff2*
     const TileSplit t = p.wide ? split_tiles(k) : TileSplit{1, 1, k, 0};
     // rows loaded together as adjoint_rows says; the residency leaves the
     // registers that keep those loads in flight
+    const Columns c = vec ? kAdjacent : p.pairs ? kApart : kSingle;
+#define FF_ADJOINT(KA, KB, R, MINB)                                                                                  \
+    (c == kAdjacent ? launch_adjoint<KA, KB, kAdjacent, R, MINB>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s) \
+     : c == kApart  ? launch_adjoint<KA, KB, kApart, R, MINB>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)    \
+                    : launch_adjoint<KA, KB, kSingle, (R > 8 ? R : 8), MINB>(p, t, A, m, n, lda, dY, lddy, out, out_ld,   \
+                                                                             rb_stride, s))
     if (k == 1 && p.gy > 1)
-        st = vec ? launch_adjoint<1, 1, 2, 16, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)
-                 : launch_adjoint<1, 1, 1, 16, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s);
+        st = FF_ADJOINT(1, 1, 16, 3);
     else if (t.ka == 1)
-        st = vec ? launch_adjoint<1, 1, 2, 8, 4>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)
-                 : launch_adjoint<1, 1, 1, 8, 4>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s);
+        st = FF_ADJOINT(1, 1, 8, 4);
     else if (t.ka == 2)
-        st = vec ? launch_adjoint<2, 1, 2, 8, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)
-                 : launch_adjoint<2, 1, 1, 8, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s);
+        st = FF_ADJOINT(2, 1, 8, 3);
     else if (t.ka == 3)
-        st = vec ? launch_adjoint<3, 2, 2, 4, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)
-                 : launch_adjoint<3, 2, 1, 8, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s);
+        st = FF_ADJOINT(3, 2, 4, 3);
     else
-        st = vec ? launch_adjoint<4, 3, 2, 4, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)
-                 : launch_adjoint<4, 3, 1, 8, 3>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s);
+        st = FF_ADJOINT(4, 3, 4, 3);
+#undef FF_ADJOINT
     if (st != FF_OK) return st;
     if (p.gy > 1) {
         const int64_t total = n * k;

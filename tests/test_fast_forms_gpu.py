@@ -127,6 +127,34 @@ def test_gemv_t_cuts(m, n, k, kind):
     same_bits(dX[:, cols], want)
 
 
+# two columns per thread, `apart` from one another: odd rows, an even row length
+# on an 8-byte address (shift 1), every width of right-hand-side tile, the last
+# columns without a partner
+@pytest.mark.parametrize("m,n,k,shift", [(1009, 2003, 33, 0), (300, 214001, 1, 0), (640, 50001, 2, 0), (701, 18301, 5, 0),
+                                         (702, 18300, 5, 1), (2401, 1027, 27, 0), (60, 270001, 4, 0)])
+@pytest.mark.parametrize("kind", ["plain", "unnormalised", "specials"])
+def test_gemv_t_columns_apart(m, n, k, shift, kind):
+    gen = torch.Generator(device=DEV).manual_seed(11)
+    store = torch.zeros(m * n + shift, 2, device=DEV)
+    A = store[shift:].view(m, n, 2)
+    A.copy_(inputs.to_ff(inputs.loguniform_f64(m * n, gen, DEV)).view(m, n, 2))
+    dY = inputs.to_ff(inputs.loguniform_f64(k * m, gen, DEV)).view(k, m, 2)
+    dY = plant(dY.cpu(), "plain" if kind == "specials" else kind, 6).to(DEV)
+    cols = np.unique(np.r_[0:4, 127:131, 255:259, n // 2:n // 2 + 3, n - 260:n - 254, n - 4:n])
+    if kind != "plain":
+        A[m // 3, cols[::2], 1] = A[m // 3, cols[::2], 0] * 0.75
+    if kind == "specials":
+        A[m // 2, int(cols[1]), 0] = float("inf")
+        A[m - 1, int(cols[3]), 0] = float("nan")
+        A[0, int(cols[5])] = torch.tensor([-0.0, 0.0], device=DEV)
+    nrb, vec = ctypes.c_int64(), ctypes.c_int()
+    _lib.call("ff_gemv_t_launch_shape", A.data_ptr(), m, n, n, k, ctypes.byref(nrb), ctypes.byref(vec))
+    assert vec.value == 0
+    dX = ff.gemv_t(A, dY).cpu().numpy()
+    want = replay.gemv_t_replay(A[:, cols].cpu().numpy(), dY.cpu().numpy(), nrb.value)
+    same_bits(dX[:, cols], want)
+
+
 # one pass, the widest single pass, two passes, the matrix-product route; even
 # and odd rows of dA; rows around the steps and the staged chunks
 @pytest.mark.parametrize("m,n,k", [(5, 6, 1), (131, 7, 1), (261, 514, 2), (129, 515, 5), (66, 36, 12), (67, 35, 13), (133, 130, 20),

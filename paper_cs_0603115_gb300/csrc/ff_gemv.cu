@@ -695,13 +695,17 @@ gemv_dA_small_kernel(const float2* __restrict__ dY, int64_t m, int64_t lddy, con
         const int n_rows = static_cast<int>(r1 - cb < kTChunk ? r1 - cb : kTChunk);
         if (cb > r0) __syncthreads();   // the previous chunk's reads are done
         bool ok = okx;
-        for (int i = threadIdx.x; i < KT * kTChunk; i += kGBlock) {
-            const int c = i / kTChunk, q = i - c * kTChunk;
-            if (q < n_rows) {
-                const float2 d = __ldg(dY + c * lddy + cb + q);
-                ok &= ffk::normalised(d);
-                sdy[c][q] = d;
-            }
+        auto stage = [&](unsigned c, unsigned q) {
+            const float2 d = __ldg(dY + c * lddy + cb + q);
+            ok &= ffk::normalised(d);
+            sdy[c][q] = d;
+        };
+        if constexpr (KT <= 5) {   // at most three rounds
+            for (int i = threadIdx.x; i < KT * kTChunk; i += kGBlock)
+                if (i % kTChunk < n_rows) stage(i / kTChunk, i % kTChunk);
+        } else {   // rounds by the rows there are: the division costs less than rounds with few of them
+            const unsigned per = n_rows, staged = KT * per;
+            for (unsigned i = threadIdx.x; i < staged; i += kGBlock) stage(i / per, i % per);
         }
         if (__syncthreads_and(ok))
             chunk(std::true_type(), cb, n_rows);
@@ -715,9 +719,14 @@ gemv_dA_small_kernel(const float2* __restrict__ dY, int64_t m, int64_t lddy, con
 // columns 1.54e12; beyond, single columns (k = 13-20: 1.61 -> 1.54e12) against
 // the GEMM kernel's 1.38-1.43e12 and the 1.35-1.53e12 of two passes over dA,
 // which they replace.  Odd row lengths take single columns throughout (4001^2,
-// k = 5: 1.46e12 terms/s; with X re-read for every element 0.59e12).
+// k = 5: 1.46e12 terms/s; with X re-read for every element 0.59e12).  Above 20
+// columns only large matrices gain over the GEMM kernel (16384^2, k = 21 / 24 / 28:
+// 3.86 / 4.34 / 5.00 -> 3.47 / 4.00 / 4.93 ms; 8192^2, k = 28 1.25 -> 1.29, 300 x 500,
+// k = 24 5.0 -> 7.4 us).
 constexpr int kDAPair = 12;
 constexpr int kDAMaxSmallK = 20;
+constexpr int kDAMaxLargeK = 28;
+constexpr double kDALarge = 268435456.0;   // values of dA
 
 // Grid: as many block rows as fill 1 to 8 waves of resident blocks, whichever
 // takes the fewest rows in turn, a wave's start counted as four rows.  One wave
@@ -914,11 +923,11 @@ ff_status ff_gemv_dA(const ff2* dY_, int64_t m, int64_t lddy, const ff2* X_, int
     if (!ffh::ok_ptr(dY_, static_cast<size_t>(m)) || !ffh::ok_ptr(X_, static_cast<size_t>(n)) || !ffh::ok_ptr(dA_, an))
         return FF_ERR_INVALID_ARG;
     if (m == 0 || n == 0) return FF_OK;
-    // beyond kDAMaxSmallK right-hand sides, dA is a matrix product op(dY) X
+    // beyond kDAMaxSmallK (kDAMaxLargeK) right-hand sides, dA is a matrix product op(dY) X
     // with dY read transposed in place: the GEMM kernel computes every
     // element with the same Mul22(dY[r, c], X[j, c]) terms in the same order
     // (bit-identical) at its higher arithmetic rate
-    if (k > kDAMaxSmallK) return ff_gemm(1, 0, m, n, k, dY_, lddy, X_, ldx, dA_, ldda, s);
+    if (k > (static_cast<double>(m) * n >= kDALarge ? kDAMaxLargeK : kDAMaxSmallK)) return ff_gemm(1, 0, m, n, k, dY_, lddy, X_, ldx, dA_, ldda, s);
     auto* dY = reinterpret_cast<const float2*>(dY_);
     auto* X = reinterpret_cast<const float2*>(X_);
     auto* dA = reinterpret_cast<float2*>(dA_);
@@ -927,7 +936,7 @@ ff_status ff_gemv_dA(const ff2* dY_, int64_t m, int64_t lddy, const ff2* X_, int
     const ff_status st = ffh::device_info(&di);
     if (st != FF_OK) return st;
     return vec && k <= kDAPair ? dA_small<kDAPair, 2>(k, dY, m, lddy, X, n, ldx, dA, ldda, di.sm_count, s)
-                               : dA_small<kDAMaxSmallK, 1>(k, dY, m, lddy, X, n, ldx, dA, ldda, di.sm_count, s);
+                               : dA_small<kDAMaxLargeK, 1>(k, dY, m, lddy, X, n, ldx, dA, ldda, di.sm_count, s);
 }
 
 ff_status ff_f64_gemv(const double* A, int64_t m, int64_t n, int64_t lda, const double* X, int64_t ldx, int64_t k,

@@ -587,9 +587,9 @@ ff_status launch_adjoint(const AdjointPlan& p, const TileSplit& t, const float2*
 // ---------------------------------------------------------------------------
 // dA = dY X^T.  Every element accumulates its k terms Mul22(dY[r, c], X[j, c])
 // in order c = 0 .. k-1 from (0, 0), so the result is the oracle's
-// left-to-right sum bit for bit.  Up to kDAMaxSmallK right-hand sides run
-// here; larger k runs as the matrix product op(dY) X on the GEMM kernel (the
-// same terms in the same order).
+// left-to-right sum bit for bit.  Up to kDAMaxSmallK right-hand sides
+// (kDAMaxLargeK for large matrices) run here; larger k runs as the matrix product
+// op(dY) X on the GEMM kernel (the same terms in the same order).
 // ---------------------------------------------------------------------------
 
 // Rows per shared-memory chunk of dY (a multiple of four).
@@ -927,7 +927,8 @@ ff_status ff_gemv_dA(const ff2* dY_, int64_t m, int64_t lddy, const ff2* X_, int
     // with dY read transposed in place: the GEMM kernel computes every
     // element with the same Mul22(dY[r, c], X[j, c]) terms in the same order
     // (bit-identical) at its higher arithmetic rate
-    if (k > (static_cast<double>(m) * n >= kDALarge ? kDAMaxLargeK : kDAMaxSmallK)) return ff_gemm(1, 0, m, n, k, dY_, lddy, X_, ldx, dA_, ldda, s);
+    if (k > (static_cast<double>(m) * n >= kDALarge ? kDAMaxLargeK : kDAMaxSmallK))
+        return ff_gemm(1, 0, m, n, k, dY_, lddy, X_, ldx, dA_, ldda, s);
     auto* dY = reinterpret_cast<const float2*>(dY_);
     auto* X = reinterpret_cast<const float2*>(X_);
     auto* dA = reinterpret_cast<float2*>(dA_);

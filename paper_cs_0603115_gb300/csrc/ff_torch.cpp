@@ -112,15 +112,16 @@ bool workspace(PyObject* cache, PyObject* key, const Where& w, size_t bytes, at:
     return held(*ws) >= bytes;
 }
 
-// The call with the GIL released, as a ctypes call makes it.
+// The call with the GIL released, as a ctypes call makes it; held again when the
+// call throws too, since what becomes of the exception touches Python.
 template <class Call>
 ff_status unlocked(Call&& call)
 {
-    ff_status st;
-    Py_BEGIN_ALLOW_THREADS
-    st = call();
-    Py_END_ALLOW_THREADS
-    return st;
+    struct Released {
+        PyThreadState* state = PyEval_SaveThread();
+        ~Released() { PyEval_RestoreThread(state); }
+    } released;
+    return call();
 }
 
 // nullptr from the body means "not taken": None.  C++ exceptions (an allocation

@@ -233,8 +233,10 @@ FF_API size_t ff_gemv_t_workspace_bytes(int64_t m, int64_t n, int64_t k);
 /* dX = A^T dY (the adjoint of ff_gemv with respect to X).  dY: m x k
  * column-major (stride lddy >= m); dX: n x k column-major (stride
  * lddx >= n), overwritten.  1 <= k <= 64.
- * Order: A is cut into row blocks (their number depends on m, n, k and the
- * device's SM count); within a block each column accumulates its rows in
+ * Order: A is cut into row blocks (their number depends on m, n, k, the access
+ * width that ff_gemv_t_launch_shape reports and the device's SM count; rows of a
+ * block plus blocks, the longest chain of additions, is at most a tenth above
+ * what min(64, m / 32) blocks give); within a block each column accumulates its rows in
  * order with Add22 from (0, 0); the blocks' partial sums (held in shared
  * memory, or in the workspace: caller-owned, ff_gemv_t_workspace_bytes, 16-byte
  * aligned) are added in row-block order.  Bit-reproducible for a given device

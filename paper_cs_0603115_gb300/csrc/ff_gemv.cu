@@ -510,7 +510,21 @@ double adjoint_cycles(const AdjointPlan& p, int64_t m, int64_t n, int64_t k, boo
     return c;
 }
 
-// The cut with the least modelled time.  Against column groups of 256 and at
+// The longest chain of additions behind one result that a cut may have: rows of a
+// row block plus row blocks.  The error of a sum grows with it, so time alone does
+// not choose.  The limit is a tenth above what row blocks of at least 32 rows, at
+// most 64 of them, give (about the least any cut reaches, 2 sqrt(m), up to 4096
+// rows): a tenth is 5% of the error, and without it the powers of two that cuts
+// come in miss the limit by a hair.  By time alone 1035 x 4196, k = 13 was cut into 4
+// blocks of 259 rows, 1.4 times the RMS error of 32 blocks of 33.
+double longest_chain(int64_t m)
+{
+    int64_t blocks = m / 32;
+    blocks = blocks < 1 ? 1 : blocks > 64 ? 64 : blocks;
+    return 1.1 * static_cast<double>(blocks + (m + blocks - 1) / blocks);
+}
+
+// The cut with the least modelled time and no longer chain than that.  Against column groups of 256 and at
 // most 64 row blocks in two launches of eight right-hand sides each, before:
 // 32768^2, k = 16: 13.8 -> 11.7 ms (with the Fast2Sum forms); 1024^2: 12.6 ->
 // 5.1 us; 10000 x 100, k = 3: 41 -> 14 us; 2001 x 3001, k = 5: 51 -> 32 us.
@@ -525,12 +539,14 @@ AdjointPlan search_adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int s
     // -> 34, 3333 x 401 11.8 -> 12.7, 1024 x 1025, k = 64 57 -> 60).
     const double values = static_cast<double>(m) * n;
     const bool pairs = !vec && n >= 1024 && values >= 2e6 && values * k >= 64e6;
+    const double chain = longest_chain(m);
     double least = -1.0;
     auto consider = [&](int cx, int64_t gy) {
         AdjointPlan p{};
         p.cx = cx;
         const int64_t rg = kGBlock / cx;
         cut_rows(m, rg * gy, &p.nrb, &p.rpb);
+        if (static_cast<double>(p.rpb + p.nrb) > chain) return;
         p.gy = (p.nrb + rg - 1) / rg;
         p.pairs = pairs;
         for (int w = 0; w < (k > 1 ? 2 : 1); ++w) {
@@ -543,11 +559,9 @@ AdjointPlan search_adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int s
         }
     };
     for (int cx = 2; cx <= kGBlock; cx *= 2) consider(cx, 1);
-    // two launches cost more than a short sum takes in one; a single right-hand
-    // side, bound by HBM, gains nothing from more row blocks (12001^2: 186 us with
-    // 28, 195 with 48)
-    if (least > 10000.0)
-        for (int64_t gy = 2; gy <= (k == 1 ? 16 : 64) && 2 * gy <= m; ++gy) consider(128, gy);
+    // two launches cost more than a short sum takes in one
+    if (least < 0.0 || least > 10000.0)
+        for (int64_t gy = 2; gy <= 64 && 2 * gy <= m; ++gy) consider(128, gy);
     return best;
 }
 

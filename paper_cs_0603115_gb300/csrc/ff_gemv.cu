@@ -468,14 +468,18 @@ inline int adjoint_rows(const AdjointPlan& p, int ka, int64_t k, bool vec)
     return ka <= 2 || !(vec || p.pairs) ? 8 : 4;
 }
 
-// Modelled cycles of a cut, fitted to a sweep of all cuts of 41 shapes (64^2 to
-// 16384^2, tall and wide, k = 1-64, even and odd rows; the cut it picks is
-// within 1.5% of the best one measured on average, at worst 12%): FP32 issue of
-// the SM with the most blocks; memory traffic (bytes per cycle of the L2, or of
-// HBM beyond it; short row segments touch more sectors than they use, and more
-// L1 lines per load); a part-filled last wave; the latency of the rows loaded
-// together; and the ordered combination, through shared memory or by a second
-// launch over the workspace.
+// Modelled cycles of a cut, fitted to sweeps of all cuts of 619 shapes (64^2 to
+// 16384^2, tall and wide, down to 2 rows and up to 10^6 columns, k = 1-64, even and
+// odd rows; of the cuts with a short enough chain it picks one within 1.2% of the
+// best measured on average, at worst 25%): FP32 issue of the SM with the most
+// blocks; memory traffic (bytes per cycle of the L2, or of HBM beyond it; short row
+// segments touch more sectors than they use, and more L1 lines per load); a part-
+// filled last wave; the latency of the rows loaded together (single columns in
+// wide tiles wait for more of them); and the ordered combination, through shared
+// memory, which every wave of blocks pays, so that a matrix wide enough to fill the
+// device is cut into few row blocks (16 x 1000000, k = 16: 290 -> 196 us, 48 x 1000000, k =
+// 5 290 -> 186, 100 x 100001, k = 5 67 -> 46, where it counted for three waves at most),
+// or by a second launch over the workspace.
 double adjoint_cycles(const AdjointPlan& p, int64_t m, int64_t n, int64_t k, bool vec, int sm_count)
 {
     const TileSplit t = p.wide ? split_tiles(k) : TileSplit{1, 1, k, 0};
@@ -499,14 +503,14 @@ double adjoint_cycles(const AdjointPlan& p, int64_t m, int64_t n, int64_t k, boo
     // right-hand side
     const double rbw = p.cx < 32 ? 32.0 / p.cx : 1.0;
     const double l1 = 0.46 * per * 8.0 * p.rpb * (std::fmax(rbw * (vec ? 1.0 : 1.4), 2.0 * e) + t.ka * rbw);
-    const double mem = std::fmax(l1, over * bytes / (8.0 * m * n > 100e6 ? 3800.0 : 6000.0));
+    const double mem = std::fmax(l1, over * bytes / (8.0 * m * n > 100e6 ? 3800.0 : 6000.0) + 8.0 * n * k / 6000.0);
     const double rounds = 1.0 + 0.36 * (std::fmin(std::ceil(waves), 3.0) - 1.0);
     double c = std::fmax(issue, mem) + 0.24 * std::fmin(issue, mem) +
-               rounds * (464.0 * ((p.rpb + rows - 1) / rows) + 1590.0);
+               rounds * (464.0 * ((p.rpb + rows - 1) / rows) + 1590.0) + (e == 1 ? 50.0 * (t.ka - 1) * rows : 0.0);
     if (p.gy > 1)
-        c += 5450.0 + 164.0 * p.nrb + 16.0 * p.nrb * n * k / 3800.0;
+        c += 14000.0 + 350.0 * p.nrb + 16.0 * p.nrb * n * k / 3800.0;
     else if (p.nrb > 1)
-        c += rounds * 59.0 * p.nrb;
+        c += 700.0 + 59.0 * p.nrb + std::fmax(waves - 0.5, 0.0) * (2000.0 + 40.0 * p.nrb);
     return c;
 }
 
@@ -536,9 +540,10 @@ AdjointPlan search_adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int s
     // dY, where the matrix gives every thread enough to do: 8191^2, k = 2 141 -> 126
     // us, 4000 x 6001, k = 5 123 -> 110, 12001^2, k = 1 190 -> 176.  Smaller or
     // narrower ones lose more to the halved number of threads (2001 x 3001, k = 5 29
-    // -> 34, 3333 x 401 11.8 -> 12.7, 1024 x 1025, k = 64 57 -> 60).
+    // -> 34, 3333 x 401 11.8 -> 12.7, 1024 x 1025, k = 64 57 -> 60), unless dX alone
+    // has enough columns for all of them (4 x 50001, k = 16 7.0 -> 5.3).
     const double values = static_cast<double>(m) * n;
-    const bool pairs = !vec && n >= 1024 && values >= 2e6 && values * k >= 64e6;
+    const bool pairs = !vec && n >= 1024 && ((values >= 2e6 && values * k >= 64e6) || static_cast<double>(n) * k >= 2e5);
     const double chain = longest_chain(m);
     double least = -1.0;
     auto consider = [&](int cx, int64_t gy) {
@@ -560,7 +565,7 @@ AdjointPlan search_adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int s
     };
     for (int cx = 2; cx <= kGBlock; cx *= 2) consider(cx, 1);
     // two launches cost more than a short sum takes in one
-    if (least < 0.0 || least > 10000.0)
+    if (least < 0.0 || least > 14000.0)
         for (int64_t gy = 2; gy <= 64 && 2 * gy <= m; ++gy) consider(128, gy);
     return best;
 }

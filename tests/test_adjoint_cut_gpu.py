@@ -60,3 +60,23 @@ def test_sums_follow_the_cut(m, n, k):
     dX = ff.gemv_t(gi.A.cuda(), gi.dY.cuda()).cpu().numpy()
     want = replay.gemv_t_replay(gi.A.numpy(), gi.dY.numpy(), nrb)
     assert (dX.view("u4") == want.view("u4")).all()
+
+
+@pytest.mark.parametrize("m,n,k", [(8, 1000000, 5), (12, 100001, 5), (16, 1000001, 2), (24, 200000, 16), (32, 200001, 5)])
+def test_wide_matrices_are_cut_into_few_row_blocks(m, n, k):
+    """The columns alone fill the device: one row block (4 to 16 before, at half the rate and less)."""
+    assert cut(m, n, k)[0] == 1
+
+
+@pytest.mark.parametrize("m,n,k", [(12, 100001, 3), (5, 70001, 4), (48, 16001, 5), (100, 20000, 2), (2, 200001, 1)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_sums_of_wide_matrices(m, n, k, offset):
+    gi = inputs.gemv(m, n, k, inputs.seed_for(4, 300 + k))
+    buf = torch.empty(m * n + 2, 2, device="cuda")
+    A = buf[offset:offset + m * n].view(m, n, 2)
+    A.copy_(gi.A)
+    nrb, _, vec = cut(m, n, k, offset)
+    assert vec == (n % 2 == 0 and offset == 0)
+    dX = ff.gemv_t(A, gi.dY.cuda()).cpu().numpy()
+    want = replay.gemv_t_replay(gi.A.numpy(), gi.dY.numpy(), nrb)
+    assert (dX.view("u4") == want.view("u4")).all()

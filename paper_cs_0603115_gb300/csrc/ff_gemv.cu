@@ -546,7 +546,7 @@ AdjointPlan search_adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int s
     const bool pairs = !vec && n >= 1024 && ((values >= 2e6 && values * k >= 64e6) || static_cast<double>(n) * k >= 2e5);
     const double chain = longest_chain(m);
     double least = -1.0;
-    auto consider = [&](int cx, int64_t gy) {
+    auto consider = [&](int cx, int64_t gy, bool wide) {
         AdjointPlan p{};
         p.cx = cx;
         const int64_t rg = kGBlock / cx;
@@ -554,41 +554,67 @@ AdjointPlan search_adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int s
         if (static_cast<double>(p.rpb + p.nrb) > chain) return;
         p.gy = (p.nrb + rg - 1) / rg;
         p.pairs = pairs;
-        for (int w = 0; w < (k > 1 ? 2 : 1); ++w) {
-            p.wide = w == 1;
-            const double c = adjoint_cycles(p, m, n, k, vec, sm_count);
-            if (least < 0.0 || c < least) {
-                least = c;
-                best = p;
-            }
+        p.wide = wide;
+        const double c = adjoint_cycles(p, m, n, k, vec, sm_count);
+        if (least < 0.0 || c < least) {
+            least = c;
+            best = p;
         }
     };
-    for (int cx = 2; cx <= kGBlock; cx *= 2) consider(cx, 1);
-    // two launches cost more than a short sum takes in one
-    if (least < 0.0 || least > 14000.0)
-        for (int64_t gy = 2; gy <= 64 && 2 * gy <= m; ++gy) consider(128, gy);
+    const int widths = k > 1 ? 2 : 1;
+    for (int cx = 2; cx <= kGBlock; cx *= 2)
+        for (int w = 0; w < widths; ++w) consider(cx, 1, w == 1);
+    // Two launches cost more than a short sum takes in one.  Of their cuts only those
+    // that just fill a number of waves are tried: of 4000 shapes 9 would take another
+    // one, for at most 7%, and the search is 5 times as fast.
+    const int64_t most = m / 2 < 64 ? m / 2 : 64;
+    if (most < 2 || (least >= 0.0 && least <= 14000.0)) return best;
+    const int64_t width = vec || pairs ? 256 : 128;
+    for (int w = 0; w < widths; ++w) {
+        const TileSplit t = w == 1 ? split_tiles(k) : TileSplit{1, 1, k, 0};
+        const int64_t blocks = (n + width - 1) / width * (t.na + t.nb);
+        const int64_t resident = static_cast<int64_t>(sm_count) * (t.ka >= 2 || k == 1 ? 3 : 4);
+        for (int64_t gy = 1; gy < most;) {
+            const int64_t waves = ((gy + 1) * blocks + resident - 1) / resident;
+            gy = waves * resident / blocks;
+            if (gy > most) gy = most;
+            consider(128, gy, w == 1);
+        }
+    }
     return best;
 }
 
-// The search takes a few microseconds and a call asks for its plan several
-// times (workspace size, then the launch): each host thread keeps the last
-// few, by sizes.
-AdjointPlan adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int sm_count)
+struct AdjointPlans {
+    AdjointPlan access8, access16;
+};
+
+// The plans of a call's sizes.  A search takes 0.2 to 1 us and a call asks for its
+// plan several times (workspace size, for both access widths, then the launch):
+// each host thread keeps those of the last sizes, four to a set.
+const AdjointPlans& adjoint_plans(int64_t m, int64_t n, int64_t k, int sm_count)
 {
     struct Entry {
-        int64_t m = -1, n, k;
-        bool vec;
-        int sm_count;
-        AdjointPlan plan;
+        int64_t m, n, k;
+        int sm_count;   // 0: empty
+        AdjointPlans plans;
     };
-    constexpr unsigned kEntries = 16;
-    static thread_local Entry kept[kEntries];
-    const uint64_t h = static_cast<uint64_t>(m) * 0x9e3779b97f4a7c15ull + static_cast<uint64_t>(n) * 0xc2b2ae3d27d4eb4full +
-                       static_cast<uint64_t>(k) * 2 + (vec ? 1 : 0);
-    Entry& e = kept[(h ^ (h >> 32)) % kEntries];
-    if (e.m != m || e.n != n || e.k != k || e.vec != vec || e.sm_count != sm_count)
-        e = Entry{m, n, k, vec, sm_count, search_adjoint_plan(m, n, k, vec, sm_count)};
-    return e.plan;
+    constexpr unsigned kSets = 16, kWays = 4;
+    static thread_local Entry kept[kSets][kWays];
+    static thread_local unsigned char oldest[kSets];
+    const uint64_t h = (static_cast<uint64_t>(m) * 0x9e3779b97f4a7c15ull + static_cast<uint64_t>(n)) * 0xc2b2ae3d27d4eb4full +
+                       static_cast<uint64_t>(k) * 0x165667b19e3779f9ull;
+    const unsigned set = static_cast<unsigned>((h >> 48) % kSets);
+    for (const Entry& e : kept[set])
+        if (e.m == m && e.n == n && e.k == k && e.sm_count == sm_count) return e.plans;
+    Entry& e = kept[set][oldest[set]++ % kWays];
+    e = Entry{m, n, k, sm_count, {search_adjoint_plan(m, n, k, false, sm_count), search_adjoint_plan(m, n, k, true, sm_count)}};
+    return e.plans;
+}
+
+inline const AdjointPlan& adjoint_plan(int64_t m, int64_t n, int64_t k, bool vec, int sm_count)
+{
+    const AdjointPlans& p = adjoint_plans(m, n, k, sm_count);
+    return vec ? p.access16 : p.access8;
 }
 
 template <int KA, int KB, Columns C, int R, int MINB>
@@ -862,8 +888,8 @@ size_t ff_gemv_t_workspace_bytes(int64_t m, int64_t n, int64_t k)
     ffh::DeviceInfo di;
     if (ffh::device_info(&di) != FF_OK) return 0;
     // the workspace must cover either access path: take the larger
-    const size_t a = adjoint_ws(adjoint_plan(m, n, k, true, di.sm_count), n, k);
-    const size_t b = adjoint_ws(adjoint_plan(m, n, k, false, di.sm_count), n, k);
+    const AdjointPlans& p = adjoint_plans(m, n, k, di.sm_count);
+    const size_t a = adjoint_ws(p.access16, n, k), b = adjoint_ws(p.access8, n, k);
     return a > b ? a : b;
 }
 

@@ -80,3 +80,23 @@ def test_sums_of_wide_matrices(m, n, k, offset):
     dX = ff.gemv_t(A, gi.dY.cuda()).cpu().numpy()
     want = replay.gemv_t_replay(gi.A.numpy(), gi.dY.numpy(), nrb)
     assert (dX.view("u4") == want.view("u4")).all()
+
+
+def test_host_time_does_not_depend_on_recent_sizes():
+    """Forty sizes in turn cost a call no more host time than one size again and again (4 us more when a
+    thread's plans held eight sizes)."""
+    import time
+    lib = _lib.load()
+    shapes = [(1000 + 211 * i, 3001 + 97 * i, 1 + i % 16) for i in range(40)]
+
+    def per_call(turn):
+        best = 1.0
+        for _ in range(7):
+            t = time.perf_counter()
+            for _ in range(10):
+                for m, n, k in turn:
+                    lib.ff_gemv_t_workspace_bytes(m, n, k)
+            best = min(best, (time.perf_counter() - t) / (10 * len(turn)))
+        return best
+
+    assert per_call(shapes) < per_call(shapes[:1] * 40) + 1e-6

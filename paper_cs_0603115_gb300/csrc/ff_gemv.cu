@@ -356,9 +356,10 @@ __device__ __forceinline__ void gemv_t_tile(const float2* __restrict__ A, int64_
                                             int cx, float2* __restrict__ out, int64_t out_ld, int64_t rb_stride,
                                             float2 (*part)[kGBlock], unsigned zero)
 {
+    const int shift = 31 - __clz(cx);   // cx is a power of two
     const int tx = threadIdx.x & (cx - 1);
-    const int ty = threadIdx.x / cx;
-    const int rg = kGBlock / cx;
+    const int ty = threadIdx.x >> shift;
+    const int rg = kGBlock >> shift;
     constexpr int E = C == kSingle ? 1 : 2;
     const int64_t j = static_cast<int64_t>(blockIdx.x + zero) * cx * E + (C == kAdjacent ? 2 * tx : tx);   // first column
     const int apart = C == kAdjacent ? 1 : cx;   // to the second one
@@ -935,12 +936,21 @@ ff_status ff_gemv_t(const ff2* A_, int64_t m, int64_t n, int64_t lda, const ff2*
     // rows loaded together as adjoint_rows says; the residency leaves the
     // registers that keep those loads in flight
     const Columns c = vec ? kAdjacent : p.pairs ? kApart : kSingle;
-#define FF_ADJOINT(KA, KB, R, MINB)                                                                                  \
+#define FF_ADJOINT_RS(KA, KB, R, RS, MINB)                                                                           \
     (c == kAdjacent ? launch_adjoint<KA, KB, kAdjacent, R, MINB>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s) \
      : c == kApart  ? launch_adjoint<KA, KB, kApart, R, MINB>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s)    \
-                    : launch_adjoint<KA, KB, kSingle, (R > 8 ? R : 8), MINB>(p, t, A, m, n, lda, dY, lddy, out, out_ld,   \
-                                                                             rb_stride, s))
-    if (k == 1 && p.gy > 1)
+                    : launch_adjoint<KA, KB, kSingle, RS, MINB>(p, t, A, m, n, lda, dY, lddy, out, out_ld, rb_stride, s))
+#define FF_ADJOINT_R(KA, KB, R, MINB) FF_ADJOINT_RS(KA, KB, R, R, MINB)
+#define FF_ADJOINT(KA, KB, R, MINB) FF_ADJOINT_RS(KA, KB, R, (R > 8 ? R : 8), MINB)
+    // Row blocks of at most three rows have no batch of rows to load together; a
+    // thread does little more than store, and more resident warps pay instead (1 x
+    // 1000000, k = 1 6.2 -> 3.9 us, k = 16 38.9 -> 30.9; 3 x 1000001, k = 2 11.4 -> 9.0).
+    if (p.rpb <= 3)
+        st = t.ka == 1   ? FF_ADJOINT_R(1, 1, 2, 6)
+             : t.ka == 2 ? FF_ADJOINT_R(2, 1, 2, 5)
+             : t.ka == 3 ? FF_ADJOINT_R(3, 2, 2, 4)
+                         : FF_ADJOINT_R(4, 3, 2, 4);
+    else if (k == 1 && p.gy > 1)
         st = FF_ADJOINT(1, 1, 16, 3);
     else if (t.ka == 1)
         st = FF_ADJOINT(1, 1, 8, 4);
@@ -951,6 +961,8 @@ ff_status ff_gemv_t(const ff2* A_, int64_t m, int64_t n, int64_t lda, const ff2*
     else
         st = FF_ADJOINT(4, 3, 4, 3);
 #undef FF_ADJOINT
+#undef FF_ADJOINT_R
+#undef FF_ADJOINT_RS
     if (st != FF_OK) return st;
     if (p.gy > 1) {
         const int64_t total = n * k;

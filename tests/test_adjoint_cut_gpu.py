@@ -100,3 +100,21 @@ def test_host_time_does_not_depend_on_recent_sizes():
         return best
 
     assert per_call(shapes) < per_call(shapes[:1] * 40) + 1e-6
+
+
+@pytest.mark.parametrize("m,n", [(1, 1), (1, 2), (1, 513), (2, 1000), (3, 257), (3, 10001), (2, 60002), (3, 2), (1, 200001)])
+@pytest.mark.parametrize("k", [1, 2, 3, 5, 9])
+@pytest.mark.parametrize("law", ["float-float", "any pairs"])
+def test_sums_of_few_rows(m, n, k, law):
+    """Row blocks of one to three rows, with operands that are normalised and that are not."""
+    if law == "any pairs":
+        g = torch.Generator().manual_seed(m + n + k)
+        A, dY = torch.randn(m, n, 2, generator=g), torch.randn(k, m, 2, generator=g)
+    else:
+        gi = inputs.gemv(m, n, k, inputs.seed_for(4, 400 + k))
+        A, dY = gi.A, gi.dY
+    nrb, rows, _ = cut(m, n, k)
+    assert rows <= 3
+    dX = ff.gemv_t(A.cuda(), dY.cuda()).cpu().numpy()
+    want = replay.gemv_t_replay(A.numpy(), dY.numpy(), nrb)
+    assert (dX.view("u4") == want.view("u4")).all()

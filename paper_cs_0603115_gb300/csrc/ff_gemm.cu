@@ -226,13 +226,16 @@ ff_status launch(bool ta, bool tb, const float2* A, const float2* B, float2* C, 
 
 // Tile choice.  Every output is one serial chain of k terms, so C is cut by
 // outputs only, and the time is that of the SM with the most tiles: measured
-// cycles per inner index with q tiles on an SM are close to  a q + b  (a: the
-// tile's outputs per lane times the cycles per term, which grow as the tile's
-// operand reuse shrinks: 25.1, 26.4, 27.6 and 30.2; b: the part of a chain's
-// latency that the few resident warps leave uncovered).  The shape with the
-// least of it runs.  500 x 300 x 700: 392 us with 64 x 64 tiles alone (40 of
-// 152 SMs busy), 82 us; 100 x 100 x 1000: 508 -> 29 us; 1024^3: 1042 -> 737
-// us; from about 2048 rows and columns the largest tile is always taken.
+// cycles with q tiles on an SM are close to  (a q + b) k + f q + g  (a: the tile's
+// outputs per lane times the cycles per term, which grow as the tile's operand
+// reuse shrinks: 25.1, 26.4, 27.6 and 30.2; b: the part of a chain's latency that
+// the few resident warps leave uncovered; f, g: a tile's first loads and its stores,
+// per tile and once).  The shape with the least of it runs; over 167 shapes with k =
+// 1 to 400 that is within 0.4% of the best one on average, at worst 10%.  500 x 300 x
+// 700: 392 us with 64 x 64 tiles alone (40 of 152 SMs busy), 82 us; 100 x 100 x 1000: 508
+// -> 29 us; 1024^3: 1042 -> 737 us; from about 2048 rows and columns the largest tile is
+// always taken.  Without f and g small k took small tiles: 1000 x 2000 x 1 19.3 -> 6.3 us
+// (the largest tile alone: 6.6), 900 x 900 x 4 10.7 -> 6.2 (7.0).
 //
 // The small tiles do few terms per inner index, so the work of one slice (its
 // loads, stores and barrier) is spread over 64 of them: 90 us at 500 x 300 x 700
@@ -243,19 +246,20 @@ using Tile16 = Tile<16, 16, 1, 2, 64, 4>;
 using Tile8 = Tile<8, 16, 1, 1, 64, 4>;
 
 template <class S>
-double cycles(int64_t m, int64_t n, int sm_count, double a, double b)
+double cycles(const Dims& d, int sm_count, double a, double b, double f, double g)
 {
-    const double tiles = static_cast<double>((m + S::BM - 1) / S::BM) * static_cast<double>((n + S::BN - 1) / S::BN);
-    return a * std::ceil(tiles / sm_count) + b;
+    const double tiles = static_cast<double>((d.m + S::BM - 1) / S::BM) * static_cast<double>((d.n + S::BN - 1) / S::BN);
+    const double q = std::ceil(tiles / sm_count), k = static_cast<double>(d.k);
+    return (a * q + b) * k + f * q + g;
 }
 
 ff_status launch_best(bool ta, bool tb, const float2* A, const float2* B, float2* C, const Dims& d, int sm_count,
                       cudaStream_t s)
 {
-    const double c64 = cycles<Tile64>(d.m, d.n, sm_count, 803.0, 45.0);
-    const double c32 = cycles<Tile32>(d.m, d.n, sm_count, 211.0, 20.0);
-    const double c16 = cycles<Tile16>(d.m, d.n, sm_count, 55.2, 28.0);
-    const double c8 = cycles<Tile8>(d.m, d.n, sm_count, 30.2, 28.0);
+    const double c64 = cycles<Tile64>(d, sm_count, 803.0, 45.0, 1600.0, 700.0);
+    const double c32 = cycles<Tile32>(d, sm_count, 211.0, 20.0, 1190.0, 0.0);
+    const double c16 = cycles<Tile16>(d, sm_count, 55.2, 28.0, 600.0, 100.0);
+    const double c8 = cycles<Tile8>(d, sm_count, 30.2, 28.0, 530.0, 200.0);
     const double best = std::fmin(std::fmin(c64, c32), std::fmin(c16, c8));
     if (best == c64) return launch<Tile64>(ta, tb, A, B, C, d, s);
     if (best == c32) return launch<Tile32>(ta, tb, A, B, C, d, s);

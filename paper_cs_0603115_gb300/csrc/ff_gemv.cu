@@ -58,7 +58,7 @@ __device__ __forceinline__ float2 shfl_down2(float2 v, int off)
 // Chunk numbers are 32-bit within segments of kSegment chunks.
 constexpr int64_t kSegment = 1 << 24;
 
-template <int KT, bool VEC, int U, bool PIPE, bool FAST>
+template <int KT, bool VEC, int U, bool PIPE, bool FAST, int LOOP = 1>
 __device__ __forceinline__ bool gemv_lane(const float2* __restrict__ Ar, const float2* __restrict__ X, int64_t n,
                                           int64_t ldx, unsigned lane, float2 (&acc)[KT])
 {
@@ -135,7 +135,7 @@ __device__ __forceinline__ bool gemv_lane(const float2* __restrict__ Ar, const f
                 }
             }
         }
-#pragma unroll 1
+#pragma unroll LOOP
         for (; t < nch; t += 32) {
             const V a = __ldcs(Av + t);
 #pragma unroll
@@ -186,35 +186,35 @@ __device__ __forceinline__ void gemv_tree_store(const float2 (&acc)[KT], int lan
     if (lane % low == 0 && c < KT) Yr[c * ldy] = ffk::ff_overflow_lo(v);
 }
 
-template <int KT, bool VEC, int U, bool PIPE>
+template <int KT, bool VEC, int U, bool PIPE, int LOOP>
 __device__ __forceinline__ void gemv_row(const float2* __restrict__ Ar, const float2* __restrict__ X, int64_t n,
                                          int64_t ldx, float2* __restrict__ Yr, int64_t ldy)
 {
     const unsigned lane = threadIdx.x & 31;
     float2 acc[KT];
-    if (gemv_lane<KT, VEC, U, PIPE, true>(Ar, X, n, ldx, lane, acc))
+    if (gemv_lane<KT, VEC, U, PIPE, true, LOOP>(Ar, X, n, ldx, lane, acc))
         gemv_lane<KT, VEC, 1, false, false>(Ar, X, n, ldx, lane, acc);
     gemv_tree_store(acc, static_cast<int>(lane), Yr, ldy);
 }
 
 // blockIdx.x: rows, one per warp; blockIdx.y: tile of right-hand sides, the
 // first `na` of them KA wide, the others KB wide.
-template <int KA, int KB, bool VEC, int U, bool PIPE, int MINB>
-__global__ void __launch_bounds__(32 * kFWarps, MINB)
+template <int KA, int KB, bool VEC, int U, bool PIPE, int MINB, int WARPS, int LOOP>
+__global__ void __launch_bounds__(32 * WARPS, MINB)
 gemv_kernel(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda, const float2* __restrict__ X,
             int64_t ldx, float2* __restrict__ Y, int64_t ldy, int na)
 {
     const unsigned zero = ffk::prior_kernel_done();
-    const int64_t r = static_cast<int64_t>(blockIdx.x + zero) * kFWarps + (threadIdx.x >> 5);
+    const int64_t r = static_cast<int64_t>(blockIdx.x + zero) * WARPS + (threadIdx.x >> 5);
     if (r >= m) return;
     const int y = blockIdx.y;
     X += zero;
     if (KA == KB || y < na) {
         const int64_t c0 = static_cast<int64_t>(y) * KA;
-        gemv_row<KA, VEC, U, PIPE>(A + r * lda, X + c0 * ldx, n, ldx, Y + c0 * ldy + r, ldy);
+        gemv_row<KA, VEC, U, PIPE, LOOP>(A + r * lda, X + c0 * ldx, n, ldx, Y + c0 * ldy + r, ldy);
     } else {
         const int64_t c0 = static_cast<int64_t>(na) * KA + static_cast<int64_t>(y - na) * KB;
-        gemv_row<KB, VEC, U, PIPE>(A + r * lda, X + c0 * ldx, n, ldx, Y + c0 * ldy + r, ldy);
+        gemv_row<KB, VEC, U, PIPE, LOOP>(A + r * lda, X + c0 * ldx, n, ldx, Y + c0 * ldy + r, ldy);
     }
 }
 
@@ -240,13 +240,13 @@ inline TileSplit split_tiles(int64_t k)
 
 inline int f64_tile_for(int64_t k) { return k >= 16 ? 16 : k >= 8 ? 8 : k >= 4 ? 4 : k >= 2 ? 2 : 1; }
 
-template <int KA, int KB, bool VEC, int U, bool PIPE, int MINB>
+template <int KA, int KB, bool VEC, int U, bool PIPE, int MINB, int WARPS = kFWarps, int LOOP = 1>
 ff_status launch_gemv(const TileSplit& t, const float2* A, int64_t m, int64_t n, int64_t lda, const float2* X,
                       int64_t ldx, float2* Y, int64_t ldy, cudaStream_t s)
 {
-    const dim3 grid(static_cast<unsigned>((m + kFWarps - 1) / kFWarps), static_cast<unsigned>(t.na + t.nb));
-    return ffh::launch_kernel(&gemv_kernel<KA, KB, VEC, U, PIPE, MINB>, grid, 32 * kFWarps, s, A, m, n, lda, X, ldx, Y,
-                              ldy, static_cast<int>(t.na));
+    const dim3 grid(static_cast<unsigned>((m + WARPS - 1) / WARPS), static_cast<unsigned>(t.na + t.nb));
+    return ffh::launch_kernel(&gemv_kernel<KA, KB, VEC, U, PIPE, MINB, WARPS, LOOP>, grid, 32 * WARPS, s, A, m, n, lda, X,
+                              ldx, Y, ldy, static_cast<int>(t.na));
 }
 
 // Chunks in flight (U) and the register budget that lets the compiler issue
@@ -257,6 +257,13 @@ ff_status launch_gemv(const TileSplit& t, const float2* A, int64_t m, int64_t n,
 // chunks and the next four of A ahead (32768^2: 1.16 ms = 7.4 TB/s, 1.21 with
 // eight and none ahead; 2000 rows and fewer prefer the latter: 300 x 20000 31.5
 // -> 21.4 us).
+// Short rows never fill four or eight chunks in flight, and serve better with one or
+// two, few registers and so twice the warps, in blocks of eight: 65536 rows, k = 1, n =
+// 64 15.2 -> 14.4 us, 100 22.2 -> 18.4, 200 41.7 -> 28.9, 1000 90 -> 82; odd rows n = 33, k = 5
+// 54.7 -> 41.9, n = 101, k = 2 32.4 -> 26.3, n = 201, k = 5 110 -> 87.  The lines lie where the
+// sweep crosses: fewer rows than 16 a quarter gain nothing, 2500 x 512 3.4 -> 3.7.  The
+// same kernel takes 8 to 12 rows a quarter at any length, where the pipelined one
+// starts a second wave that it does not fill (5000 x 16384: 128 -> 110 us; 8000 156, 152).
 // Few rows leave SMs idle under a wide tile, since a row is one warp's: below
 // one warp per SM quarter the right-hand sides get a warp each (400 x 2000, k =
 // 4: 6.9 us in pairs, 5.7 singly), below two they go in pairs (800 x 2000, k = 4:
@@ -270,8 +277,25 @@ ff_status gemv_forward(const float2* A, int64_t m, int64_t n, int64_t lda, const
     const TileSplit t = split_tiles(k);
     const int64_t warps = m * ((k + 3) / 4);
     const int64_t quarters = 4 * static_cast<int64_t>(sm_count);
-    if (VEC && k == 1 && warps >= 4 * quarters)
-        return launch_gemv<1, 1, VEC, 4, true, 0>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+    if constexpr (VEC) {
+        if (k == 1 && n <= 128 && m >= 16 * quarters)
+            return launch_gemv<1, 1, true, 1, false, 0, 8>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+        if (k == 1 && n > 128 && m > 8 * quarters && (m <= 12 * quarters || n <= 400 || (n <= 2048 && m >= 24 * quarters)))
+            return launch_gemv<1, 1, true, 1, false, 0, 8, 2>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+        if (k == 1 && m >= 4 * quarters)
+            return launch_gemv<1, 1, true, 4, true, 0>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+    } else if (n <= 128 && m >= 16 * quarters) {
+        if (k == 1) return launch_gemv<1, 1, false, 1, false, 0, 8>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+        if (k == 2) return launch_gemv<2, 1, false, 1, false, 0, 8>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+        if (t.ka == 3) return launch_gemv<3, 2, false, 1, false, 0, 8>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+        return launch_gemv<4, 3, false, 1, false, 0, 8>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+    } else if (n <= 256 && k == 1 && m >= 16 * quarters) {
+        return launch_gemv<1, 1, false, 4, false, 5, 8>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+    } else if (n <= 256 && m >= 64 * quarters) {
+        if (k == 2) return launch_gemv<2, 1, false, 2, false, 0, 8>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+        if (t.ka == 3) return launch_gemv<3, 2, false, 2, false, 0, 8>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+        return launch_gemv<4, 3, false, 2, false, 0, 8>(t, A, m, n, lda, X, ldx, Y, ldy, s);
+    }
     if (k == 1 || warps < quarters)
         return launch_gemv<1, 1, VEC, 8, false, 4>({1, 1, k, 0}, A, m, n, lda, X, ldx, Y, ldy, s);
     if (k == 2 || warps < 2 * quarters)

@@ -331,7 +331,7 @@ typedef struct ff_batch_instance {
 /* Launch configuration of the batched kernel: threads per block (128, 256
  * or 512), values per thread per tile (pairs_per_thread: 8 .. 128, tile =
  * block x pairs_per_thread values), resident blocks per SM that walk the tiles
- * (0 = a block per tile; for many tiles of GEMV instances alone, as many
+ * (0 = a block per tile; for many large tiles of GEMV instances alone, as many
  * resident blocks as fit) and two-value chunks per input loaded ahead of use
  * (unroll: 2 or 4; 0 = 4). */
 typedef struct ff_tune {

@@ -633,6 +633,9 @@ ff_status ff_batch_plan_create(const ff_batch_instance* inst, int count, const f
             // four rows per warp at a time, rpw groups of four per warp per tile
             const int64_t warps = tune.block / 32;
             int64_t rpw = gemv_tile / (4 * warps * (b.n > 0 ? b.n : 1));
+            // spread over all the tile's warps where the matrix has fewer rows than that
+            // (20000 matrices of 32 x 32: 257 -> 72 us, of 8 x 8: 68 -> 51)
+            rpw = std::min<int64_t>(rpw, (b.m + 4 * warps - 1) / (4 * warps));
             rpw = rpw < 1 ? 1 : (rpw > 16 ? 16 : rpw);
             d.rows_per_warp = static_cast<int32_t>(rpw);
             const int64_t rows_per_tile = 4 * warps * rpw;
@@ -691,17 +694,19 @@ ff_status ff_batch_plan_create(const ff_batch_instance* inst, int count, const f
     // free, so long and short tiles balance, and a block that computes always has
     // one that loads beside it.  Blocks that stay and walk the tiles in fixed steps
     // took 350 us for 1024 dot and AXPY instances of up to 1e6 values, 322 this way.
-    // GEMV tiles alone, more than four per resident block, are better walked by
+    // Large GEMV tiles alone, more than four per resident block, are better walked by
     // resident blocks with the tile counter: 300 matrices of up to 3000 x 3000 186
     // us, 188 with a block per tile; fewer save the counter's clearing (1000 of up to
-    // 100 x 100: 17.6 -> 15.2).
+    // 100 x 100: 17.6 -> 15.2), and small ones would wait for the counter, their tile
+    // and their instance one after the other (20000 of 16 to 300: 442, 434; 1000 of 100 to
+    // 300: 65, 61).
     int64_t grid = 0x7fffffff;
     if (tune.blocks_per_sm > 0) {
         grid = static_cast<int64_t>(di.sm_count) * tune.blocks_per_sm;
     } else if (p->only_gemv_rows) {
         const int occ = ffh::occupancy(reinterpret_cast<const void*>(kernel_for(*var, *p)), tune.block);
         const int64_t resident = static_cast<int64_t>(di.sm_count) * (occ > 0 ? occ : 1);
-        if (p->ntiles > 4 * resident) grid = resident;
+        if (p->ntiles > 4 * resident && total >= 12000 * p->ntiles) grid = resident;
     }
     if (grid > p->ntiles) grid = p->ntiles > 0 ? p->ntiles : 1;
     p->grid = static_cast<unsigned>(grid);

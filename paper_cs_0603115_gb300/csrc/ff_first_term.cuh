@@ -10,8 +10,8 @@
 
 namespace ffk {
 
-// Add22((+0, +0), t) bit for bit for a finite normalised t (every mul22_fast
-// result of normalised operands is one, or not finite): the Add22 theorem's
+// Add22((+0, +0), t) bit for bit for a finite normalised t (every mul22 result is
+// one, or not finite, and so is every mul22_fast result of normalised operands): the Add22 theorem's
 // steps reduce to r = th (+) 0, s = tl (+) 0 and a closing sum that returns (r,
 // s): th - r = +0 (the tie branch when th = +-0, which forces tl = +-0), the
 // zero operand's low part adds nothing.  "(+) 0" does what the full sequence

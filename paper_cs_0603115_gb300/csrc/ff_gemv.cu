@@ -672,8 +672,9 @@ constexpr int kTChunk = 128;
 // one 16-byte read gives two rows of one right-hand side.  Every element is
 // Add22((0, 0), term_0), then Add22 of terms 1 .. KT-1, in order.
 // The chunk's dY and the threads' X are checked once, in the staging barrier:
-// a chunk whose values are all normalised takes the Fast2Sum forms (and the
-// first step from (0, 0) in two additions), any other the full ones.
+// a chunk whose values are all normalised takes the Fast2Sum forms, any other the
+// full ones; the first of several steps from (0, 0) takes two additions either way,
+// since a finite product is normalised whatever its operands are.
 // Threads past the last column work on the last one and do not store, so that
 // every thread reaches the barriers.
 template <int KT, int E>
@@ -726,7 +727,7 @@ gemv_dA_small_kernel(const float2* __restrict__ dY, int64_t m, int64_t lddy, con
                 for (int e = 0; e < E; ++e) {
                     const float2 t = FAST ? ffk::mul22_fast(d[r], x[c][e]) : ffk::mul22(d[r], x[c][e]);
                     if (c == 0)
-                        a[r][e] = FAST ? ffk::add22_from_zero_fast(t) : ffk::add22(make_float2(0.0f, 0.0f), t);
+                        a[r][e] = FAST || KT > 1 ? ffk::add22_from_zero_fast(t) : ffk::add22(make_float2(0.0f, 0.0f), t);
                     else
                         a[r][e] = FAST ? ffk::add22_fast(a[r][e], t) : ffk::add22(a[r][e], t);
                 }

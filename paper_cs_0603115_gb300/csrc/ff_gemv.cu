@@ -373,6 +373,23 @@ __device__ __forceinline__ bool gemv_t_sums(const float2* __restrict__ Aj, int a
     return bad;
 }
 
+// The full forms, out of line: inlined, they took registers from the fast ones as
+// soon as they loaded more than one row ahead (8192^2, k = 1, pairs that are not
+// normalised: 246 us with one row, 171 with four; float-float operands 0.3% faster).
+// A check for them within the fast loops cost those 4 to 7%.
+template <int KT, Columns C, int R>
+__device__ __noinline__ void gemv_t_sums_full(const float2* Aj, int apart, int64_t lda, const float2* dY, int64_t lddy,
+                                              int64_t r0, int64_t r1, float2 (*sums)[C == kSingle ? 1 : 2])
+{
+    constexpr int E = C == kSingle ? 1 : 2;
+    float2 acc[KT][E];
+    gemv_t_sums<KT, C, R, false>(Aj, apart, lda, dY, lddy, r0, r1, acc);
+#pragma unroll
+    for (int c = 0; c < KT; ++c)
+#pragma unroll
+        for (int e = 0; e < E; ++e) sums[c][e] = acc[c][e];
+}
+
 // The block's tile of KT right-hand sides; see gemv_t_kernel.
 template <int KT, Columns C, int R>
 __device__ __forceinline__ void gemv_t_tile(const float2* __restrict__ A, int64_t m, int64_t n, int64_t lda,
@@ -394,8 +411,18 @@ __device__ __forceinline__ void gemv_t_tile(const float2* __restrict__ A, int64_
     float2 acc[KT][E];
     const bool active = j < n && rb < nrb;
     const int step = second ? apart : 0;
-    if (active && gemv_t_sums<KT, C, R, true>(A + j, step, lda, dY, lddy, r0, r1, acc))
-        gemv_t_sums<KT, C, 1, false>(A + j, step, lda, dY, lddy, r0, r1, acc);
+    if (active && gemv_t_sums<KT, C, R, true>(A + j, step, lda, dY, lddy, r0, r1, acc)) {
+        if constexpr (R > 2) {
+            float2 sums[KT][E];
+            gemv_t_sums_full<KT, C, 4>(A + j, step, lda, dY, lddy, r0, r1, sums);
+#pragma unroll
+            for (int c = 0; c < KT; ++c)
+#pragma unroll
+                for (int e = 0; e < E; ++e) acc[c][e] = sums[c][e];
+        } else {
+            gemv_t_sums<KT, C, 1, false>(A + j, step, lda, dY, lddy, r0, r1, acc);
+        }
+    }
     if (rg == 1 || gridDim.y > 1) {
         if (!active) return;
         float2* o = out + rb * rb_stride + j;

@@ -684,9 +684,9 @@ ff_status launch_adjoint(const AdjointPlan& p, const TileSplit& t, const float2*
 // ---------------------------------------------------------------------------
 // dA = dY X^T.  Every element accumulates its k terms Mul22(dY[r, c], X[j, c])
 // in order c = 0 .. k-1 from (0, 0), so the result is the oracle's
-// left-to-right sum bit for bit.  Up to kDAMaxSmallK right-hand sides
-// (kDAMaxLargeK for large matrices) run here; larger k runs as the matrix product
-// op(dY) X on the GEMM kernel (the same terms in the same order).
+// left-to-right sum bit for bit.  Up to max_dA right-hand sides run here; larger k
+// runs as the matrix product op(dY) X on the GEMM kernel (the same terms in the same
+// order).
 // ---------------------------------------------------------------------------
 
 // Rows per shared-memory chunk of dY (a multiple of four).
@@ -818,13 +818,18 @@ gemv_dA_small_kernel(const float2* __restrict__ dY, int64_t m, int64_t lddy, con
 // the GEMM kernel's 1.38-1.43e12 and the 1.35-1.53e12 of two passes over dA,
 // which they replace.  Odd row lengths take single columns throughout (4001^2,
 // k = 5: 1.46e12 terms/s; with X re-read for every element 0.59e12).  Above 20
-// columns only large matrices gain over the GEMM kernel (16384^2, k = 21 / 24 / 28:
-// 3.86 / 4.34 / 5.00 -> 3.47 / 4.00 / 4.93 ms; 8192^2, k = 28 1.25 -> 1.29, 300 x 500,
-// k = 24 5.0 -> 7.4 us).
+// columns it depends on the size, over 28 shapes of 10^6 to 4 10^8 values, square, tall
+// and wide: k = 21-24 take 0.88-0.96 of the GEMM kernel's time from 4 10^6 values on (1.04-
+// 1.07 at 10^6), k = 26 0.94-1.00 from 6.5 10^7 on (0.99-1.02 from 2.5 to 4.2 10^7), k = 28
+// 0.98-1.06; narrow ones leave threads of their last block idle (100 columns, k = 24 1.11).
 constexpr int kDAPair = 12;
-constexpr int kDAMaxSmallK = 20;
-constexpr int kDAMaxLargeK = 28;
-constexpr double kDALarge = 268435456.0;   // values of dA
+constexpr int kDAMax = 26;
+
+inline int max_dA(int64_t m, int64_t n)
+{
+    const double values = static_cast<double>(m) * n;
+    return n < 1024 || values < 4e6 ? 20 : values < 6.5e7 ? 24 : kDAMax;
+}
 
 // Grid: as many block rows as fill 1 to 8 waves of resident blocks, whichever
 // takes the fewest rows in turn, a wave's start counted as four rows.  One wave
@@ -1032,11 +1037,10 @@ ff_status ff_gemv_dA(const ff2* dY_, int64_t m, int64_t lddy, const ff2* X_, int
     if (!ffh::ok_ptr(dY_, static_cast<size_t>(m)) || !ffh::ok_ptr(X_, static_cast<size_t>(n)) || !ffh::ok_ptr(dA_, an))
         return FF_ERR_INVALID_ARG;
     if (m == 0 || n == 0) return FF_OK;
-    // beyond kDAMaxSmallK (kDAMaxLargeK) right-hand sides, dA is a matrix product op(dY) X
-    // with dY read transposed in place: the GEMM kernel computes every
-    // element with the same Mul22(dY[r, c], X[j, c]) terms in the same order
-    // (bit-identical) at its higher arithmetic rate
-    if (k > (static_cast<double>(m) * n >= kDALarge ? kDAMaxLargeK : kDAMaxSmallK))
+    // beyond max_dA right-hand sides, dA is a matrix product op(dY) X with dY read
+    // transposed in place: the GEMM kernel computes every element with the same
+    // Mul22(dY[r, c], X[j, c]) terms in the same order (bit-identical)
+    if (k > max_dA(m, n))
         return ff_gemm(1, 0, m, n, k, dY_, lddy, X_, ldx, dA_, ldda, s);
     auto* dY = reinterpret_cast<const float2*>(dY_);
     auto* X = reinterpret_cast<const float2*>(X_);
@@ -1046,7 +1050,7 @@ ff_status ff_gemv_dA(const ff2* dY_, int64_t m, int64_t lddy, const ff2* X_, int
     const ff_status st = ffh::device_info(&di);
     if (st != FF_OK) return st;
     return vec && k <= kDAPair ? dA_small<kDAPair, 2>(k, dY, m, lddy, X, n, ldx, dA, ldda, di.sm_count, s)
-                               : dA_small<kDAMaxLargeK, 1>(k, dY, m, lddy, X, n, ldx, dA, ldda, di.sm_count, s);
+                               : dA_small<kDAMax, 1>(k, dY, m, lddy, X, n, ldx, dA, ldda, di.sm_count, s);
 }
 
 ff_status ff_f64_gemv(const double* A, int64_t m, int64_t n, int64_t lda, const double* X, int64_t ldx, int64_t k,

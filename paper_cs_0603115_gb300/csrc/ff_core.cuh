@@ -79,7 +79,8 @@ __device__ __forceinline__ float2 fast2sum(float a, float b)
 // ---------------------------------------------------------------------------
 // Mul22 and Add22 with Fast2Sum in place of their closing Add12: 9 + 13 = 22
 // instructions per accumulated term instead of 12 + 16 = 28, for the kernels
-// bound by FP32 issue.  Same bits as mul22 / add22 under these conditions:
+// bound by FP32 issue.  Sums of such terms have the bits of sums of mul22 / add22
+// under these conditions:
 //
 // mul22_fast: |t3| <= |t1| (or t1 = t3 = 0).  Both forms then give
 //   RN(t1 + t3) and its exact error.  A pair whose sum rounds to its high
@@ -94,8 +95,14 @@ __device__ __forceinline__ float2 fast2sum(float a, float b)
 //   never below that of s, which is Fast2Sum's condition.
 // A closing sum that is exact leaves a normalised result, so accumulating
 // mul22_fast terms from (0, 0) (or from any Add22 result) stays inside the
-// conditions.  Signs of zeros: neither t3 nor s is ever -0 where t1 or r is
-// zero, and an exact closing sum gives lo = +0 both ways.
+// conditions.  Signs of zeros: the closings differ where their second operand is
+// -0 (Add12 leaves lo = +0, Fast2Sum -0).  mul22_fast meets that when products
+// underflow: (-2^-100, -2^-130) times (2^-100, 2^-130) gives t3 = -0 and (-0, -0) for
+// mul22's (-0, +0).  So its result is only ever an addend, not to be stored itself.
+// A sum from (+0, +0) never holds -0 and does not see the sign of a zero added to
+// it: P, the sum's own high part when both are zero, is not -0, so neither P - r
+// nor anything added to that is; s, never -0, closes alike both ways.
+// (add22_from_zero_fast adds +0, with the same effect.)
 // Infinities and NaN: any step with a non-finite operand gives (NaN, NaN) in
 // both forms.  The one difference is a step that overflows to hi = +-inf: lo
 // is NaN with Add12 and -+inf with Fast2Sum; a further add22 / add22_fast

@@ -33,6 +33,9 @@
  *     with n == 0 writes (0, 0) to its result.
  *   - Aliasing.  An elementwise output may be exactly one of its inputs
  *     (in place); any other overlap is undefined.
+ *   - Operands.  Any pairs are accepted.  The matrix products, GEMVs and
+ *     adjoints are fastest on normalised ones (hi + lo rounds to hi, as every
+ *     result of this library does) and give the documented sums on all.
  *   - Results.  Every elementwise result is the exact op sequence of the
  *     cited algorithm in binary32 round-to-nearest-even, with subnormals
  *     kept: bit-for-bit reproducible.  Reductions follow the fixed tree order

@@ -6,8 +6,8 @@
 // Layouts: A is m x n row-major (row stride lda); X, dX are n x k and Y, dY
 // are m x k, all column-major (column strides ldx, lddx, ldy, lddy).
 //
-// ff_gemv: one warp per row, four rows per block, a tile of up to four right-
-// hand sides per warp, all tiles in one launch.  Lane l walks the row in two-
+// ff_gemv: one warp per row, four rows per block (eight where rows are short), a
+// tile of up to four right-hand sides per warp, all tiles in one launch.  Lane l walks the row in two-
 // column steps (j = 2l + 64t, 16-byte loads of A and of each column of X; single
 // columns j = l + 32t on 8-byte access) and keeps one float-float accumulator
 // per right-hand side.  The 32 lane accumulators are combined by a shuffle-down
@@ -40,7 +40,7 @@ namespace {
 constexpr int kGBlock = 256;
 constexpr int kGWarps = kGBlock / 32;
 constexpr int kMaxK = 64;
-constexpr int kFWarps = 4;   // rows (one per warp) of a forward block
+constexpr int kFWarps = 4;   // rows (one per warp) of a forward block, unless its launch says otherwise
 
 __device__ __forceinline__ float2 shfl_down2(float2 v, int off)
 {
